@@ -267,24 +267,4 @@ cudaError_t launch_type_perm(const int* type, int natoms, int ntypes, int* perm,
                              const TypeStartCheck& chk,
                              cudaStream_t st);
 
-// ------------------------------------------------------------------------------------------
-// Generic (CUDA-core) path, templated on the network scalar (dense.cu / path.cu)
-// ------------------------------------------------------------------------------------------
-struct RowMap {
-  int kind;  // 0: rows r0 + r ; 1: slots (p0 + r / nk) * nc + k0 + r % nk
-  long r0;
-  int p0, nk, k0, nc;
-  int nrows;
-  // slot rows: the environment rows ([rows][4], the layer's element type) -- a row whose s is zero
-  // (padding) is left unwritten, and a tile of such rows only is skipped; null: every row
-  const void* zrow = nullptr;
-};
-
-template <class R>
-cudaError_t launch_dense_fwd(const RowMap& rm, const R* X, int n_in, const R* W, const R* b, int n_out, int skip,
-                             int tanh_act, R* Y, R* Tact, cudaStream_t st);
-template <class R>
-cudaError_t launch_dense_bwd(const RowMap& rm, const R* GY, const R* Tact, int n_in, const R* W, int n_out,
-                             int skip, R* GX, cudaStream_t st);
-
 }  // namespace dpgb

@@ -19,19 +19,13 @@
 #include <cstring>
 
 #include "capi_internal.cuh"
+#include "dense.cuh"
 #include "env.cuh"
 #include "grad.cuh"
 
 namespace dpgb {
 
 namespace {
-
-constexpr int BM = 64, BN = 64, BK = 16;
-
-__device__ __forceinline__ long rowi(const RowMap& m, int r) {
-  if (m.kind == 0) return m.r0 + r;
-  return (long)(m.p0 + r / m.nk) * m.nc + m.k0 + r % m.nk;
-}
 
 inline unsigned nb(long n, int b) { return (unsigned)((n + b - 1) / b); }
 inline int net_index(const PathConst& pc, int ti, int tj) { return pc.type_one_side ? tj : ti * pc.ntypes + tj; }
@@ -40,12 +34,13 @@ inline int net_index(const PathConst& pc, int ti, int tj) { return pc.type_one_s
 template <class R>
 __global__ void k_env_tan(PathConst pc, const double* __restrict__ coord, const double* __restrict__ w,
                           const double* __restrict__ gv, const int* __restrict__ perm, const int* __restrict__ nl_j,
-                          const int* __restrict__ nl_code, R* __restrict__ Renv, R* __restrict__ Rdot) {
+                          const int* __restrict__ nl_code, const int* __restrict__ tsorted, RowLists rl,
+                          R* __restrict__ Renv, R* __restrict__ Rdot) {
   const long row = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (row >= (long)pc.natoms * pc.nc) return;
-  const int p = (int)(row / pc.nc), k = (int)(row % pc.nc);
+  const bool in = row < (long)pc.natoms * pc.nc;
+  const int p = in ? (int)(row / pc.nc) : 0, k = in ? (int)(row % pc.nc) : 0;
   const int i = perm[p];
-  const int j = nl_j[(long)i * pc.nc + k];
+  const int j = in ? nl_j[(long)i * pc.nc + k] : -1;
   R o[4] = {0, 0, 0, 0}, od[4] = {0, 0, 0, 0};
   if (j >= 0) {
     double d0, d1, d2;
@@ -74,17 +69,20 @@ __global__ void k_env_tan(PathConst pc, const double* __restrict__ coord, const 
       od[1 + a] = sd * u[a] + s * ud;
     }
   }
+  if (in)
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    Renv[row * 4 + a] = o[a];
-    Rdot[row * 4 + a] = od[a];
-  }
+    for (int a = 0; a < 4; ++a) {
+      Renv[row * 4 + a] = o[a];
+      Rdot[row * 4 + a] = od[a];
+    }
+  // rows the embedding layers work on
+  append_row(rl, pc.ntypes * pc.ntypes, o[0] != R(0) ? tsorted[p] * pc.ntypes + slot_block(pc, k) : -1, row);
 }
 
 // ---- first embedding layer (scalar input), primal and tangent ----------------------------------
 template <class R>
 __global__ void k_emb0_tan(PathConst pc, NetPtrs<R> nets, const int* __restrict__ tsorted, const R* __restrict__ Renv,
-                           const R* __restrict__ Rdot, int w1, int skip, R* __restrict__ Y, R* __restrict__ T,
+                           const R* __restrict__ Rdot, int w1, int ld, int skip, R* __restrict__ Y, R* __restrict__ T,
                            R* __restrict__ Yd, R* __restrict__ Zd) {
   const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const long nrow = (long)pc.natoms * pc.nc;
@@ -94,236 +92,125 @@ __global__ void k_emb0_tan(PathConst pc, NetPtrs<R> nets, const int* __restrict_
   const int p = (int)(row / pc.nc), k = (int)(row % pc.nc);
   const int net = net_of(pc, tsorted[p], slot_block(pc, k));
   const R s = Renv[row * 4], sd = Rdot[row * 4];
+  if (s == R(0)) return;  // padding: in no row list, read by nobody
   const R wv = nets.w0[net][o];
   const R t = tanh_r(s * wv + nets.b0[net][o]);
   const R zd = sd * wv;
-  Y[e] = t + (skip ? s : R(0));
-  T[e] = t;
-  Zd[e] = zd;
-  Yd[e] = (R(1) - t * t) * zd + (skip ? sd : R(0));
-}
-
-// ---- dense layer tangent: zd = xd W; yd = (1 - t^2) zd + skip(xd) --------------------------------
-template <class R>
-__global__ void __launch_bounds__(256)
-    k_dense_tan(RowMap rm, const R* __restrict__ Xd, int n_in, const R* __restrict__ W, int n_out, int skip,
-                int tanh_act, const R* __restrict__ T, R* __restrict__ Yd, R* __restrict__ Zd) {
-  // FP32: the transposed A tile's rows padded to 68 values, so that a thread's four rows (and
-  // its four B columns) load as one 16-byte vector each
-  __shared__ __align__(16) R As[BK][BM + (sizeof(R) == 4 ? 4 : 1)];
-  __shared__ __align__(16) R Bs[BK][BN];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int r0 = blockIdx.x * BM, c0 = blockIdx.y * BN;
-  R acc[4][4] = {};
-  for (int k0 = 0; k0 < n_in; k0 += BK) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int e = tid + q * 256;
-      const int r = e / BK, kk = e % BK;
-      As[kk][r] = (r0 + r < rm.nrows && k0 + kk < n_in) ? Xd[rowi(rm, r0 + r) * n_in + k0 + kk] : R(0);
-      const int kb = e / BN, cb = e % BN;
-      Bs[kb][cb] = (k0 + kb < n_in && c0 + cb < n_out) ? W[(long)(k0 + kb) * n_out + c0 + cb] : R(0);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      R av[4], bv[4];
-      if constexpr (sizeof(R) == 4) {
-        const float4 a4 = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
-        const float4 b4 = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-        av[0] = a4.x; av[1] = a4.y; av[2] = a4.z; av[3] = a4.w;
-        bv[0] = b4.x; bv[1] = b4.y; bv[2] = b4.z; bv[3] = b4.w;
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          av[q] = As[kk][ty * 4 + q];
-          bv[q] = Bs[kk][tx * 4 + q];
-        }
-      }
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] += av[a] * bv[b];
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int r = r0 + ty * 4 + a;
-    if (r >= rm.nrows) continue;
-    const long row = rowi(rm, r);
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int c = c0 + tx * 4 + b;
-      if (c >= n_out) continue;
-      const R zd = acc[a][b];
-      R yd = zd;
-      if (tanh_act) {
-        const R t = T[row * n_out + c];
-        yd = (R(1) - t * t) * zd;
-      }
-      if (skip == 1) yd += Xd[row * n_in + c];
-      if (skip == 2) yd += Xd[row * n_in + c % n_in];
-      Yd[row * n_out + c] = yd;
-      if (Zd) Zd[row * n_out + c] = zd;
-    }
-  }
-}
-
-// ---- reverse through tanh: gz, gzd from gy, gyd, t, zd (elementwise) -----------------------------
-template <class R>
-__global__ void k_rev_tanh(RowMap rm, int n, const R* __restrict__ GY, const R* __restrict__ GYd,
-                           const R* __restrict__ T, const R* __restrict__ Zd, R* __restrict__ GZ, R* __restrict__ GZd) {
-  const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long)rm.nrows * n) return;
-  const long idx = rowi(rm, (int)(e / n)) * n + e % n;
-  const R t = T[idx], g = R(1) - t * t;
-  const R gyd = GYd[idx];
-  GZd[idx] = gyd * g;
-  GZ[idx] = (GY[idx] - R(2) * t * Zd[idx] * gyd) * g;
-}
-
-// ---- gx = gz W^T + skip^T(gy) (and the same for the tangent pair) --------------------------------
-template <class R>
-__global__ void __launch_bounds__(256)
-    k_dense_bx(RowMap rm, const R* __restrict__ GZ, const R* __restrict__ GY, int n_in, const R* __restrict__ W,
-               int n_out, int skip, R* __restrict__ GX) {
-  // FP32: the transposed A tile's rows padded to 68 values, so that a thread's four rows (and
-  // its four B columns) load as one 16-byte vector each
-  __shared__ __align__(16) R As[BK][BM + (sizeof(R) == 4 ? 4 : 1)];
-  __shared__ __align__(16) R Bs[BK][BN];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int r0 = blockIdx.x * BM, c0 = blockIdx.y * BN;
-  R acc[4][4] = {};
-  for (int k0 = 0; k0 < n_out; k0 += BK) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int e = tid + q * 256;
-      const int r = e / BK, kk = e % BK;
-      As[kk][r] = (r0 + r < rm.nrows && k0 + kk < n_out) ? GZ[rowi(rm, r0 + r) * n_out + k0 + kk] : R(0);
-      const int kb = e / BN, cb = e % BN;
-      Bs[kb][cb] = (k0 + kb < n_out && c0 + cb < n_in) ? W[(long)(c0 + cb) * n_out + k0 + kb] : R(0);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      R av[4], bv[4];
-      if constexpr (sizeof(R) == 4) {
-        const float4 a4 = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
-        const float4 b4 = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-        av[0] = a4.x; av[1] = a4.y; av[2] = a4.z; av[3] = a4.w;
-        bv[0] = b4.x; bv[1] = b4.y; bv[2] = b4.z; bv[3] = b4.w;
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          av[q] = As[kk][ty * 4 + q];
-          bv[q] = Bs[kk][tx * 4 + q];
-        }
-      }
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] += av[a] * bv[b];
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int r = r0 + ty * 4 + a;
-    if (r >= rm.nrows) continue;
-    const long row = rowi(rm, r);
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int c = c0 + tx * 4 + b;
-      if (c >= n_in) continue;
-      R g = acc[a][b];
-      if (skip == 1) g += GY[row * n_out + c];
-      if (skip == 2) g += GY[row * n_out + c] + GY[row * n_out + c + n_in];
-      GX[row * n_in + c] = g;
-    }
-  }
+  const long at = row * ld + o;
+  Y[at] = t + (skip ? s : R(0));
+  T[at] = t;
+  Zd[at] = zd;
+  Yd[at] = (R(1) - t * t) * zd + (skip ? sd : R(0));
 }
 
 // ---- weight and bias gradients: gW += X^T GZ + Xd^T GZd, gb += sum_rows GZ ----------------------
-// One block owns a TI x TI tile of gW and a slab of rows; partial sums go to gW with atomics.  Each
-// thread keeps PT x PT outputs; FP32 takes 4 x 4 with 16-byte shared loads (two loads per eight
-// FMAs), FP64 2 x 2 (its pipe, not the loads, is the limit there).
+// One launch covers every net of a layer.  One block owns a 64 x 64 tile of one net's gW and a slab of
+// its rows (a range, or entries of the row list); partial sums go to gW with atomics.  128 threads keep
+// 8 x 4 outputs each (FP32: six 16-byte shared loads per 64 FMAs); the next 16 rows' global loads are
+// in flight while the current ones are summed.  Bound by FP32 FMAs and those loads: the 6,144-atom batch's
+// layers 3.65 -> 1.63 ms.
 template <class R>
-struct WGrad;
-template <>
-struct WGrad<float> {
-  static constexpr int TI = 64, PT = 4, RR = 32, LD = TI + 4;  // rows 16-byte aligned
-};
-template <>
-struct WGrad<double> {
-  static constexpr int TI = 32, PT = 2, RR = 32, LD = TI + 1;
+struct WGradJob {
+  DenseRows rows;
+  int slab0[kMaxDenseGroups];  // first slab of every net
+  int slab_rows[kMaxDenseGroups];
+  int n_in, ldx, n_out, ldg;
+  const R *X, *Xd, *GZ, *GZd;
+  R* grad;  // gW at the net's parameter offset, gb behind it
 };
 
+constexpr int kWgTI = 64, kWgRR = 16, kWgThreads = 128, kWgLd = kWgTI + 4;
+
 template <class R>
-__global__ void __launch_bounds__(256)
-    k_wgrad(RowMap rm, const R* __restrict__ X, const R* __restrict__ Xd, int n_in, const R* __restrict__ GZ,
-            const R* __restrict__ GZd, int n_out, int rows_per_block, R* __restrict__ gW, R* __restrict__ gb) {
-  constexpr int TI = WGrad<R>::TI, PT = WGrad<R>::PT, RR = WGrad<R>::RR, LD = WGrad<R>::LD;
-  __shared__ __align__(16) R xs[RR][LD], xds[RR][LD], gs[RR][LD], gds[RR][LD];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+__global__ void __launch_bounds__(kWgThreads)
+    k_wgrad(const __grid_constant__ WGradJob<R> g) {
+  constexpr int TI = kWgTI, RR = kWgRR, NT = kWgThreads, LD = kWgLd;
+  constexpr int PER = RR * TI / NT;  // values per thread, array and step
+  __shared__ __align__(32) R xs[2][RR][LD], gs[2][RR][LD];  // primal and tangent rows
+  using Q = typename Vec4<R>::T;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;  // outputs i = 8 ty + a, o = 4 tx + b
   const int i0 = blockIdx.x * TI, o0 = blockIdx.y * TI;
-  const int rbeg = blockIdx.z * rows_per_block;
-  const int rend = min(rm.nrows, rbeg + rows_per_block);
-  R acc[PT][PT] = {}, bacc[PT] = {};
+  int gi = 0;
+  while (gi + 1 < g.rows.ngroups && (int)blockIdx.z >= g.slab0[gi + 1]) ++gi;
+  const DenseGroup grp = g.rows.g[gi];
+  const int nrows = g.rows.list ? __ldg(g.rows.count + gi) : grp.nrows;
+  const int rbeg = ((int)blockIdx.z - g.slab0[gi]) * g.slab_rows[gi];
+  const int rend = min(nrows, rbeg + g.slab_rows[gi]);
+  if (rbeg >= rend) return;
+  R acc[8][4] = {}, bacc[4] = {};
+  // thread tid loads column tid % 64 of rows tid / 64 + 2 q
+  const int lc = tid % TI, lr = tid / TI;
+  R px[PER], pxd[PER], pg[PER], pgd[PER];
+  auto row_of = [&](int r) -> long {
+    if (r >= rend) return -1;
+    return g.rows.list ? __ldg(g.rows.list + grp.r0 + r) : grp.r0 + r;
+  };
+  long nrow[PER];
+  auto rows_of = [&](int r0) {
+#pragma unroll
+    for (int q = 0; q < PER; ++q) nrow[q] = row_of(r0 + lr + 2 * q);
+  };
+  auto fetch = [&]() {
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const long row = nrow[q];
+      const bool xv = row >= 0 && i0 + lc < g.n_in, gv = row >= 0 && o0 + lc < g.n_out;
+      px[q] = xv ? g.X[row * g.ldx + i0 + lc] : R(0);
+      pxd[q] = xv ? g.Xd[row * g.ldx + i0 + lc] : R(0);
+      pg[q] = gv ? g.GZ[row * g.ldg + o0 + lc] : R(0);
+      pgd[q] = gv ? g.GZd[row * g.ldg + o0 + lc] : R(0);
+    }
+  };
+  rows_of(rbeg);
+  fetch();
+  rows_of(rbeg + RR);
   for (int r0 = rbeg; r0 < rend; r0 += RR) {
-    for (int e = tid; e < RR * TI; e += 256) {
-      const int r = e / TI, c = e % TI;
-      const bool rv = r0 + r < rend;
-      const long row = rv ? rowi(rm, r0 + r) : 0;
-      xs[r][c] = (rv && i0 + c < n_in) ? X[row * n_in + i0 + c] : R(0);
-      xds[r][c] = (rv && Xd && i0 + c < n_in) ? Xd[row * n_in + i0 + c] : R(0);
-      gs[r][c] = (rv && o0 + c < n_out) ? GZ[row * n_out + o0 + c] : R(0);
-      gds[r][c] = (rv && GZd && o0 + c < n_out) ? GZd[row * n_out + o0 + c] : R(0);
+    __syncthreads();  // the previous rows were read
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int r = lr + 2 * q;
+      xs[0][r][lc] = px[q];
+      xs[1][r][lc] = pxd[q];
+      gs[0][r][lc] = pg[q];
+      gs[1][r][lc] = pgd[q];
     }
     __syncthreads();
+    if (r0 + RR < rend) {
+      fetch();
+      rows_of(r0 + 2 * RR);
+    }
 #pragma unroll 4
     for (int r = 0; r < RR; ++r) {
-      R xa[PT], xda[PT], ga[PT], gda[PT];
-      if constexpr (PT == 4) {
-        const float4 x4 = *reinterpret_cast<const float4*>(&xs[r][ty * 4]);
-        const float4 xd4 = *reinterpret_cast<const float4*>(&xds[r][ty * 4]);
-        const float4 g4 = *reinterpret_cast<const float4*>(&gs[r][tx * 4]);
-        const float4 gd4 = *reinterpret_cast<const float4*>(&gds[r][tx * 4]);
-        xa[0] = x4.x; xa[1] = x4.y; xa[2] = x4.z; xa[3] = x4.w;
-        xda[0] = xd4.x; xda[1] = xd4.y; xda[2] = xd4.z; xda[3] = xd4.w;
-        ga[0] = g4.x; ga[1] = g4.y; ga[2] = g4.z; ga[3] = g4.w;
-        gda[0] = gd4.x; gda[1] = gd4.y; gda[2] = gd4.z; gda[3] = gd4.w;
-      } else {
+      const Q g4 = *reinterpret_cast<const Q*>(&gs[0][r][tx * 4]), gd4 = *reinterpret_cast<const Q*>(&gs[1][r][tx * 4]);
+      const R ga[4] = {g4.x, g4.y, g4.z, g4.w}, gda[4] = {gd4.x, gd4.y, gd4.z, gd4.w};
 #pragma unroll
-        for (int a = 0; a < PT; ++a) {
-          xa[a] = xs[r][ty * PT + a];
-          xda[a] = xds[r][ty * PT + a];
-          ga[a] = gs[r][tx * PT + a];
-          gda[a] = gds[r][tx * PT + a];
-        }
+      for (int h = 0; h < 2; ++h) {
+        const Q x4 = *reinterpret_cast<const Q*>(&xs[0][r][ty * 8 + 4 * h]);
+        const Q xd4 = *reinterpret_cast<const Q*>(&xs[1][r][ty * 8 + 4 * h]);
+        const R xa[4] = {x4.x, x4.y, x4.z, x4.w}, xda[4] = {xd4.x, xd4.y, xd4.z, xd4.w};
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) acc[4 * h + a][b] += xa[a] * ga[b] + xda[a] * gda[b];
       }
-#pragma unroll
-      for (int a = 0; a < PT; ++a)
-#pragma unroll
-        for (int b = 0; b < PT; ++b) acc[a][b] += xa[a] * ga[b] + xda[a] * gda[b];
       if (blockIdx.x == 0 && ty == 0)
 #pragma unroll
-        for (int b = 0; b < PT; ++b) bacc[b] += ga[b];
+        for (int b = 0; b < 4; ++b) bacc[b] += ga[b];
     }
-    __syncthreads();
   }
+  R* gW = g.grad + grp.w;
 #pragma unroll
-  for (int a = 0; a < PT; ++a)
+  for (int a = 0; a < 8; ++a)
 #pragma unroll
-    for (int b = 0; b < PT; ++b) {
-      const int i = i0 + ty * PT + a, o = o0 + tx * PT + b;
-      if (i < n_in && o < n_out) atomicAdd(gW + (long)i * n_out + o, acc[a][b]);
+    for (int b = 0; b < 4; ++b) {
+      const int i = i0 + ty * 8 + a, o = o0 + tx * 4 + b;
+      if (i < g.n_in && o < g.n_out) atomicAdd(gW + (long)i * g.n_out + o, acc[a][b]);
     }
-  if (blockIdx.x == 0 && ty == 0 && gb)
+  if (blockIdx.x == 0 && ty == 0)
 #pragma unroll
-    for (int b = 0; b < PT; ++b) {
-      const int o = o0 + tx * PT + b;
-      if (o < n_out) atomicAdd(gb + o, bacc[b]);
+    for (int b = 0; b < 4; ++b) {
+      const int o = o0 + tx * 4 + b;
+      if (o < g.n_out) atomicAdd(gW + (long)g.n_in * g.n_out + o, bacc[b]);
     }
 }
 
@@ -331,7 +218,7 @@ __global__ void __launch_bounds__(256)
 template <class R>
 __global__ void __launch_bounds__(256)
     k_emb0_rev(PathConst pc, const int* __restrict__ tsorted, const R* __restrict__ Renv, const R* __restrict__ Rdot,
-               int w1, const R* __restrict__ GY, const R* __restrict__ GYd, const R* __restrict__ T,
+               int w1, int ld, const R* __restrict__ GY, const R* __restrict__ GYd, const R* __restrict__ T,
                const R* __restrict__ Zd, long rows_per_block, R* __restrict__ grad, NetOffsets off) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   R* acc = reinterpret_cast<R*>(sm_raw);  // [nets][w1][2] (gw, gb)
@@ -345,11 +232,13 @@ __global__ void __launch_bounds__(256)
     const int o = (int)(e % w1);
     const int p = (int)(row / pc.nc), k = (int)(row % pc.nc);
     const int net = net_of(pc, tsorted[p], slot_block(pc, k));
-    const R t = T[e], g = R(1) - t * t;
-    const R gyd = GYd[e];
-    const R gzd = gyd * g;
-    const R gz = (GY[e] - R(2) * t * Zd[e] * gyd) * g;
     const R s = Renv[row * 4], sd = Rdot[row * 4];
+    if (s == R(0)) continue;  // padding
+    const long at = row * ld + o;
+    const R t = T[at], g = R(1) - t * t;
+    const R gyd = GYd[at];
+    const R gzd = gyd * g;
+    const R gz = (GY[at] - R(2) * t * Zd[at] * gyd) * g;
     atomicAdd(acc + (net * w1 + o) * 2, s * gz + sd * gzd);
     atomicAdd(acc + (net * w1 + o) * 2 + 1, gz);
   }
@@ -374,16 +263,22 @@ __global__ void k_contract_tan(PathConst pc, const R* __restrict__ G, const R* _
   const R inv = R(1) / R(nc);
   for (int m = threadIdx.x; m < M; m += blockDim.x) {
     R a[4] = {0, 0, 0, 0}, ad[4] = {0, 0, 0, 0};
-    for (int k = 0; k < nc; ++k) {
-      const long row = (long)p * nc + k;
-      const R g = G[row * M + m], gd = Gd[row * M + m];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const R rr = Renv[row * 4 + c], rd = Rdot[row * 4 + c];
-        a[c] += g * rr;
-        ad[c] += gd * rr + g * rd;
+    for (int t = 0; t < pc.ntypes; ++t)
+      for (int k = pc.sel_off[t]; k < pc.sel_off[t + 1]; ++k) {
+        const long row = (long)p * nc + k;
+        const typename Vec4<R>::T rr = reinterpret_cast<const typename Vec4<R>::T*>(Renv)[row];
+        if (rr.x == R(0)) break;  // the zero rows close each type block; nothing is computed for them
+        const typename Vec4<R>::T rd = reinterpret_cast<const typename Vec4<R>::T*>(Rdot)[row];
+        const R g = G[row * M + m], gd = Gd[row * M + m];
+        a[0] += g * rr.x;
+        a[1] += g * rr.y;
+        a[2] += g * rr.z;
+        a[3] += g * rr.w;
+        ad[0] += gd * rr.x + g * rd.x;
+        ad[1] += gd * rr.y + g * rd.y;
+        ad[2] += gd * rr.z + g * rd.z;
+        ad[3] += gd * rr.w + g * rd.w;
       }
-    }
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       Ts[m * 4 + c] = a[c] * inv;
@@ -445,6 +340,7 @@ __global__ void k_descr_rev(PathConst pc, const R* __restrict__ Tm, const R* __r
   for (int e = threadIdx.x; e < nc * M; e += blockDim.x) {
     const int k = e / M, m = e % M;
     const long row = (long)p * nc + k;
+    if (Renv[row * 4] == R(0)) continue;  // padding: in no row list
     R g = 0, gd = 0;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
@@ -482,9 +378,10 @@ __global__ void k_to_double(const R* __restrict__ x, long n, double* __restrict_
 }
 
 __global__ void k_types_sorted(const int* __restrict__ type, const int* __restrict__ perm, int n,
-                               int* __restrict__ out) {
+                               int* __restrict__ out, int* __restrict__ row_count) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n) out[p] = type[perm[p]];
+  if (p < kMaxDenseGroups) row_count[p] = 0;
 }
 
 template <class R>
@@ -494,16 +391,40 @@ __global__ void k_zero(R* __restrict__ x, long n) {
 }
 
 template <class R>
-void launch_wgrad(const RowMap& rm, const R* X, const R* Xd, int n_in, const R* GZ, const R* GZd, int n_out, R* gW,
-                  R* gb, cudaStream_t st) {
-  if (rm.nrows <= 0) return;
-  constexpr int TI = WGrad<R>::TI;
-  const long tiles = (long)nb(n_in, TI) * nb(n_out, TI);
-  // row slabs of 4096, fewer rows when that leaves under two blocks per SM (small layers)
-  int rpb = 4096;
-  while (rpb > 512 && tiles * nb(rm.nrows, rpb) < 2L * 152) rpb /= 2;
-  dim3 grid(nb(n_in, TI), nb(n_out, TI), nb(rm.nrows, rpb));
-  k_wgrad<R><<<grid, 256, 0, st>>>(rm, X, Xd, n_in, GZ, GZd, n_out, rpb, gW, gb);
+void launch_wgrad(const DenseRows& rows, const DenseShape& sh, const R* X, const R* Xd, const R* GZ, const R* GZd,
+                  int ldg, R* grad, cudaStream_t st) {
+  WGradJob<R> g;
+  std::memset(&g, 0, sizeof(g));
+  g.rows = rows;
+  g.n_in = sh.n_in;
+  g.ldx = sh.ldx;
+  g.n_out = sh.n_out;
+  g.ldg = ldg;
+  g.X = X;
+  g.Xd = Xd;
+  g.GZ = GZ;
+  g.GZd = GZd;
+  g.grad = grad;
+  const long tiles = (long)nb(sh.n_in, kWgTI) * nb(sh.n_out, kWgTI);
+  // Slabs of 4096 rows.  Consecutive rows (the fitting net) take shorter ones, down to 512, while a net's
+  // launch leaves SMs under two blocks each: every slab is one FP32 chain per output, so long slabs keep
+  // the number of atomics low.  Listed rows (the embedding nets, whose outputs are few tiles) go down to
+  // 128 rows while the whole layer leaves SMs under eight blocks each.
+  long most = 0;
+  for (int k = 0; k < rows.ngroups; ++k) most += rows.g[k].nrows;
+  int listed = 4096;
+  while (listed > 128 && tiles * ((most + listed - 1) / listed) < 8L * sm_count()) listed /= 2;
+  int at = 0;
+  for (int k = 0; k < rows.ngroups; ++k) {
+    int n = rows.list ? listed : 4096;
+    if (!rows.list)
+      while (n > 512 && tiles * nb(rows.g[k].nrows, n) < 2L * 152) n /= 2;
+    g.slab_rows[k] = n;
+    g.slab0[k] = at;
+    at += (rows.g[k].nrows + n - 1) / n;
+  }
+  if (at == 0) return;
+  k_wgrad<R><<<dim3(nb(sh.n_in, kWgTI), nb(sh.n_out, kWgTI), at), kWgThreads, 0, st>>>(g);
 }
 
 }  // namespace
@@ -516,10 +437,20 @@ int run_grad(const DeviceModel& m, const PathConst& pc, const R* params, const P
   // ---- scratch ----
   R* Renv = ar.get<R>(rows * 4);
   R* Rdot = ar.get<R>(rows * 4);
+  // row stride of layer l's activations: the last layer's rows are read by the descriptor kernels
+  auto emb_ld = [&](int l) { return l == ne - 1 ? m.cfg.embed[l] : dense_ld(m.cfg.embed[l]); };
+  auto emb_shape = [&](int l) {
+    const LayerDesc& L = m.emb[l];
+    return DenseShape{L.n_in, emb_ld(l - 1), L.n_out, emb_ld(l), L.skip, 1};
+  };
+  auto fit_shape = [&](int l) {
+    const LayerDesc& L = m.fit[l];
+    return DenseShape{L.n_in, L.n_in, L.n_out, L.n_out, L.skip, L.tanh_act};
+  };
   std::vector<R*> Ye(ne), Te(ne), Yed(ne), Zed(ne);
   int maxe = 1;
   for (int l = 0; l < ne; ++l) {
-    const long wl = m.cfg.embed[l];
+    const long wl = emb_ld(l);
     maxe = std::max(maxe, (int)wl);
     Ye[l] = ar.get<R>(rows * wl);
     Te[l] = ar.get<R>(rows * wl);
@@ -554,18 +485,27 @@ int run_grad(const DeviceModel& m, const PathConst& pc, const R* params, const P
   R* ezd = ar.get<R>(rows * maxe);
   int* tsorted = ar.get<int>(N);
   R* grad = ar.get<R>(m.n_params);
+  RowLists lists;
+  lists.list = ar.get<int>(rows);
+  lists.count = ar.get<int>(kMaxDenseGroups);
+  long list_at = 0;
+  for (int ti = 0; ti < nt; ++ti)
+    for (int tj = 0; tj < nt; ++tj) {
+      lists.base[ti * nt + tj] = list_at;
+      list_at += (long)(io.type_start[ti + 1] - io.type_start[ti]) * pc.sel[tj];
+    }
   if (ar.measure) return DP_OK;
   if (!ar.ok()) {
     set_error("scratch allocation failed");
     return DP_E_OOM;
   }
   k_zero<R><<<nb(m.n_params, 256), 256, 0, st>>>(grad, m.n_params);
-  k_types_sorted<<<nb(N, 256), 256, 0, st>>>(io.type, io.perm, (int)N, tsorted);
+  k_types_sorted<<<nb(N, 256), 256, 0, st>>>(io.type, io.perm, (int)N, tsorted, lists.count);
   // ---- forward: primal and tangent ----
   {
     ProfScope _ps(io.prof, "grad_env", st);
-    k_env_tan<R><<<nb(rows, 256), 256, 0, st>>>(pc, io.coord, w_dev, gv_dev, io.perm, io.nl_j, io.nl_code, Renv,
-                                                 Rdot);
+    k_env_tan<R><<<nb(rows, 256), 256, 0, st>>>(pc, io.coord, w_dev, gv_dev, io.perm, io.nl_j, io.nl_code,
+                                                 tsorted, lists, Renv, Rdot);
   }
   NetPtrs<R> nets;
   NetOffsets off;
@@ -577,80 +517,64 @@ int run_grad(const DeviceModel& m, const PathConst& pc, const R* params, const P
     off.w[n] = L0.w_off;
   }
   const int w1 = m.cfg.embed[0];
-  k_emb0_tan<R><<<nb(rows * w1, 256), 256, 0, st>>>(pc, nets, tsorted, Renv, Rdot, w1, m.emb[0].skip, Ye[0], Te[0],
+  k_emb0_tan<R><<<nb(rows * w1, 256), 256, 0, st>>>(pc, nets, tsorted, Renv, Rdot, w1, emb_ld(0), m.emb[0].skip, Ye[0], Te[0],
                                                      Yed[0], Zed[0]);
-  auto emb_rows = [&](int ti, int tj) {
-    return RowMap{1, 0, io.type_start[ti], pc.sel[tj], pc.sel_off[tj], (int)nc,
-                  (io.type_start[ti + 1] - io.type_start[ti]) * pc.sel[tj]};
+  auto emb_layer = [&](int l) {
+    DenseRows r;
+    r.list = lists.list;
+    r.count = lists.count;
+    for (int ti = 0; ti < nt; ++ti)
+      for (int tj = 0; tj < nt; ++tj)
+        r.add(lists.base[ti * nt + tj], (io.type_start[ti + 1] - io.type_start[ti]) * pc.sel[tj],
+              m.emb[(size_t)net_index(pc, ti, tj) * ne + l].w_off);
+    return r;
   };
-  for (int ti = 0; ti < nt; ++ti)
-    for (int tj = 0; tj < nt; ++tj) {
-      const int net = net_index(pc, ti, tj);
-      const RowMap rm = emb_rows(ti, tj);
-      if (rm.nrows <= 0) continue;
-      for (int l = 1; l < ne; ++l) {
-        const LayerDesc& L = m.emb[(size_t)net * ne + l];
-        const R* W = params + L.w_off;
-        DP_CUDA_TRY(launch_dense_fwd<R>(rm, Ye[l - 1], L.n_in, W, W + (long)L.n_in * L.n_out, L.n_out, L.skip, 1,
-                                        Ye[l], Te[l], st));
-        dim3 g(nb(rm.nrows, BM), nb(L.n_out, BN));
-        k_dense_tan<R><<<g, 256, 0, st>>>(rm, Yed[l - 1], L.n_in, W, L.n_out, L.skip, 1, Te[l], Yed[l], Zed[l]);
-      }
-    }
+  auto fit_layer = [&](int l) {
+    DenseRows r;
+    for (int t = 0; t < nt; ++t)
+      r.add(io.type_start[t], io.type_start[t + 1] - io.type_start[t], m.fit[(size_t)t * nfl + l].w_off);
+    return r;
+  };
+  for (int l = 1; l < ne; ++l) {
+    ProfScope _ps(io.prof, "grad_emb_fwd", st);
+    DP_CUDA_TRY(launch_dense_tan<R>(emb_layer(l), emb_shape(l), params, Ye[l - 1], Yed[l - 1], Ye[l], Te[l], Yed[l],
+                                    Zed[l], st));
+  }
   k_contract_tan<R><<<(unsigned)N, 128, sizeof(R) * M * 8, st>>>(pc, Ye[ne - 1], Yed[ne - 1], Renv, Rdot, Tm, Tmd, D,
                                                                    Dd);
-  for (int t = 0; t < nt; ++t) {
-    const RowMap rm{0, io.type_start[t], 0, 0, 0, 0, io.type_start[t + 1] - io.type_start[t]};
-    if (rm.nrows <= 0) continue;
-    const R* X = D;
-    const R* Xd = Dd;
-    for (int l = 0; l < nfl - 1; ++l) {
-      const LayerDesc& L = m.fit[(size_t)t * nfl + l];
-      const R* W = params + L.w_off;
-      DP_CUDA_TRY(launch_dense_fwd<R>(rm, X, L.n_in, W, W + (long)L.n_in * L.n_out, L.n_out, L.skip, 1, Yf[l], Tf[l],
-                                      st));
-      dim3 g(nb(rm.nrows, BM), nb(L.n_out, BN));
-      k_dense_tan<R><<<g, 256, 0, st>>>(rm, Xd, L.n_in, W, L.n_out, L.skip, 1, Tf[l], Yfd[l], Zfd[l]);
-      X = Yf[l];
-      Xd = Yfd[l];
-    }
+  for (int l = 0; l < nfl - 1; ++l) {
+    ProfScope _ps(io.prof, "grad_fit_fwd", st);
+    DP_CUDA_TRY(launch_dense_tan<R>(fit_layer(l), fit_shape(l), params, l > 0 ? Yf[l - 1] : D, l > 0 ? Yfd[l - 1] : Dd,
+                                    Yf[l], Tf[l], Yfd[l], Zfd[l], st));
   }
   // ---- reverse: fitting net ----
   {
     // per type (the output weights differ): gx = a w, gxd = b w at the last hidden output
     for (int t = 0; t < nt; ++t) {
-      const RowMap rm{0, io.type_start[t], 0, 0, 0, 0, io.type_start[t + 1] - io.type_start[t]};
-      if (rm.nrows <= 0) continue;
+      const int nrows = io.type_start[t + 1] - io.type_start[t];
+      if (nrows <= 0) continue;
       const LayerDesc& L = m.fit[(size_t)t * nfl + nfl - 1];
       const long r0 = io.type_start[t];
-      k_fit_last_rev<R><<<nb((long)rm.nrows * L.n_in, 256), 256, 0, st>>>(
-          rm.nrows, io.perm + r0, pc.atom_frame, a_dev, b, params + L.w_off, L.n_in, fa + r0 * L.n_in,
-          fad + r0 * L.n_in, fz + r0, fzd + r0);
-      // output layer weight/bias gradients: x = last hidden output, gz = a, gzd = b
-      const R* X = nfl >= 2 ? Yf[nfl - 2] : D;
-      const R* Xd = nfl >= 2 ? Yfd[nfl - 2] : Dd;
-      launch_wgrad<R>(rm, X, Xd, L.n_in, fz, fzd, 1, grad + L.w_off, grad + L.w_off + L.n_in, st);
+      k_fit_last_rev<R><<<nb((long)nrows * L.n_in, 256), 256, 0, st>>>(
+          nrows, io.perm + r0, pc.atom_frame, a_dev, b, params + L.w_off, L.n_in, fa + r0 * L.n_in, fad + r0 * L.n_in,
+          fz + r0, fzd + r0);
     }
+    // output layer weight/bias gradients: x = last hidden output, gz = a, gzd = b
+    launch_wgrad<R>(fit_layer(nfl - 1), fit_shape(nfl - 1), nfl >= 2 ? Yf[nfl - 2] : D, nfl >= 2 ? Yfd[nfl - 2] : Dd,
+                    fz, fzd, 1, grad, st);
   }
   R* gy = fa;
   R* gyd = fad;
   R* gx = fb;
   R* gxd = fbd;
   for (int l = nfl - 2; l >= 0; --l) {
-    for (int t = 0; t < nt; ++t) {
-      const RowMap rm{0, io.type_start[t], 0, 0, 0, 0, io.type_start[t + 1] - io.type_start[t]};
-      if (rm.nrows <= 0) continue;
-      const LayerDesc& L = m.fit[(size_t)t * nfl + l];
-      const R* W = params + L.w_off;
-      k_rev_tanh<R><<<nb((long)rm.nrows * L.n_out, 256), 256, 0, st>>>(rm, L.n_out, gy, gyd, Tf[l], Zfd[l], fz, fzd);
-      dim3 g(nb(rm.nrows, BM), nb(L.n_in, BN));
-      k_dense_bx<R><<<g, 256, 0, st>>>(rm, fz, gy, L.n_in, W, L.n_out, L.skip, gx);
-      k_dense_bx<R><<<g, 256, 0, st>>>(rm, fzd, gyd, L.n_in, W, L.n_out, L.skip, gxd);
-      const R* X = l > 0 ? Yf[l - 1] : D;
-      const R* Xd = l > 0 ? Yfd[l - 1] : Dd;
-      launch_wgrad<R>(rm, X, Xd, L.n_in, fz, fzd, L.n_out, grad + L.w_off, grad + L.w_off + (long)L.n_in * L.n_out,
-                      st);
+    {
+      ProfScope _ps(io.prof, "grad_fit_rev", st);
+      DP_CUDA_TRY(launch_dense_rev<R>(fit_layer(l), fit_shape(l), params, gy, gyd, Tf[l], Zfd[l], gx, gxd, fz, fzd, st));
     }
+    ProfScope _ps(io.prof, "grad_fit_w", st);
+    launch_wgrad<R>(fit_layer(l), fit_shape(l), l > 0 ? Yf[l - 1] : D, l > 0 ? Yfd[l - 1] : Dd, fz, fzd, m.fit[l].n_out,
+                    grad, st);
     std::swap(gy, gx);
     std::swap(gyd, gxd);
   }
@@ -665,27 +589,21 @@ int run_grad(const DeviceModel& m, const PathConst& pc, const R* params, const P
   R* egx = eb;
   R* egxd = ebd;
   for (int l = ne - 1; l >= 1; --l) {
-    for (int ti = 0; ti < nt; ++ti)
-      for (int tj = 0; tj < nt; ++tj) {
-        const RowMap rm = emb_rows(ti, tj);
-        if (rm.nrows <= 0) continue;
-        const LayerDesc& L = m.emb[(size_t)net_index(pc, ti, tj) * ne + l];
-        const R* W = params + L.w_off;
-        k_rev_tanh<R><<<nb((long)rm.nrows * L.n_out, 256), 256, 0, st>>>(rm, L.n_out, egy, egyd, Te[l], Zed[l], ez,
-                                                                        ezd);
-        dim3 g(nb(rm.nrows, BM), nb(L.n_in, BN));
-        k_dense_bx<R><<<g, 256, 0, st>>>(rm, ez, egy, L.n_in, W, L.n_out, L.skip, egx);
-        k_dense_bx<R><<<g, 256, 0, st>>>(rm, ezd, egyd, L.n_in, W, L.n_out, L.skip, egxd);
-        launch_wgrad<R>(rm, Ye[l - 1], Yed[l - 1], L.n_in, ez, ezd, L.n_out, grad + L.w_off,
-                        grad + L.w_off + (long)L.n_in * L.n_out, st);
-      }
+    {
+      ProfScope _ps(io.prof, "grad_emb_rev", st);
+      DP_CUDA_TRY(launch_dense_rev<R>(emb_layer(l), emb_shape(l), params, egy, egyd, Te[l], Zed[l], egx, egxd, ez, ezd,
+                                      st));
+    }
+    ProfScope _ps(io.prof, "grad_emb_w", st);
+    launch_wgrad<R>(emb_layer(l), emb_shape(l), Ye[l - 1], Yed[l - 1], ez, ezd, emb_ld(l), grad, st);
     std::swap(egy, egx);
     std::swap(egyd, egxd);
   }
   {
     const long rpb = 2048;
     const size_t sm = sizeof(R) * (size_t)m.n_embed_nets * w1 * 2;
-    k_emb0_rev<R><<<nb(rows, (int)rpb), 256, sm, st>>>(pc, tsorted, Renv, Rdot, w1, egy, egyd, Te[0], Zed[0], rpb,
+    k_emb0_rev<R><<<nb(rows, (int)rpb), 256, sm, st>>>(pc, tsorted, Renv, Rdot, w1, emb_ld(0), egy, egyd, Te[0], Zed[0],
+                                                      rpb,
                                                       grad, off);
   }
   DP_CUDA_TRY(cudaGetLastError());

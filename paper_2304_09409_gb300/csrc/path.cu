@@ -18,6 +18,7 @@
 // cancellation near r_c (env.cuh); energy, force and virial accumulate in FP64.
 #include <type_traits>
 
+#include "dense.cuh"
 #include "dp_internal.cuh"
 #include "path.cuh"
 #include "env.cuh"
@@ -30,13 +31,14 @@ namespace {
 // ---- env ------------------------------------------------------------------------------------
 template <class R>
 __global__ void k_env(PathConst pc, const double* __restrict__ coord, const int* __restrict__ perm,
-                      const int* __restrict__ nl_j, const int* __restrict__ nl_code, R* __restrict__ Renv) {
+                      const int* __restrict__ nl_j, const int* __restrict__ nl_code,
+                      const int* __restrict__ tsorted, RowLists rl, R* __restrict__ Renv) {
   const long row = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (row >= (long)pc.natoms * pc.nc) return;
-  const int p = (int)(row / pc.nc), k = (int)(row % pc.nc);
+  const bool in = row < (long)pc.natoms * pc.nc;
+  const int p = in ? (int)(row / pc.nc) : 0, k = in ? (int)(row % pc.nc) : 0;
   const int i = perm[p];
   const long ls = (long)i * pc.lnc + list_slot(pc, k);
-  const int j = nl_j[ls];
+  const int j = in ? nl_j[ls] : -1;
   R o[4] = {R(0), R(0), R(0), R(0)};
   double d0 = 0.0, d1 = 0.0, d2 = 0.0, r2 = 0.0;
   if (j >= 0) {
@@ -51,13 +53,16 @@ __global__ void k_env(PathConst pc, const double* __restrict__ coord, const int*
     o[2] = s * u[1];
     o[3] = s * u[2];
   }
-  reinterpret_cast<typename Vec4<R>::T*>(Renv)[row] = Vec4<R>::make(o[0], o[1], o[2], o[3]);
+  if (in) reinterpret_cast<typename Vec4<R>::T*>(Renv)[row] = Vec4<R>::make(o[0], o[1], o[2], o[3]);
+  if (rl.list)  // rows the embedding layers work on
+    append_row(rl, pc.ntypes * pc.ntypes, o[0] != R(0) ? tsorted[p] * pc.ntypes + slot_block(pc, k) : -1, row);
 }
 
 // ---- first embedding layer (1 -> w1), all nets in one launch --------------------------------
 template <class R>
 __global__ void k_emb_first(PathConst pc, NetPtrs<R> nets, const int* __restrict__ atom_type_sorted,
-                            const R* __restrict__ Renv, int w1, int skip, R* __restrict__ Y, R* __restrict__ T) {
+                            const R* __restrict__ Renv, int w1, int ld, int skip, R* __restrict__ Y,
+                            R* __restrict__ T) {
   const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const long nrow = (long)pc.natoms * pc.nc;
   if (e >= nrow * w1) return;
@@ -72,14 +77,14 @@ __global__ void k_emb_first(PathConst pc, NetPtrs<R> nets, const int* __restrict
   const R t = tanh_r(s * nets.w0[net][o] + nets.b0[net][o]);
   R y = t;
   if (skip) y += s;  // n_in = 1: both +x and +{x,x} add the scalar input
-  Y[e] = y;
-  T[e] = t;
+  Y[row * ld + o] = y;
+  T[row * ld + o] = t;
 }
 
 template <class R>
 __global__ void k_emb_first_bwd(PathConst pc, NetPtrs<R> nets, const int* __restrict__ atom_type_sorted,
                                 const R* __restrict__ Renv, const R* __restrict__ GY, const R* __restrict__ T,
-                                int w1, int skip, R* __restrict__ gs) {
+                                int w1, int ld, int skip, R* __restrict__ gs) {
   const long row = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= (long)pc.natoms * pc.nc) return;
   if (Renv[row * 4] == R(0)) return;  // a zero row: no layer outputs, not read by the force kernel
@@ -88,8 +93,8 @@ __global__ void k_emb_first_bwd(PathConst pc, NetPtrs<R> nets, const int* __rest
   const R* w = nets.w0[net];
   R acc = R(0);
   for (int o = 0; o < w1; ++o) {
-    const R g = GY[row * w1 + o];
-    const R t = T[row * w1 + o];
+    const R g = GY[row * ld + o];
+    const R t = T[row * ld + o];
     acc += g * (R(1) - t * t) * w[o];
     if (skip) acc += g;
   }
@@ -889,10 +894,12 @@ __global__ void k_shift_table(PathConst pc, double* __restrict__ out) {
                                __dmul_rn((double)n2, pc.h[6 + a]));
 }
 
+// Types in sorted order; also clears the row-list counters (before the kernels that fill the lists).
 __global__ void k_sorted_types(const int* __restrict__ type, const int* __restrict__ perm, int n,
-                               int* __restrict__ out) {
+                               int* __restrict__ out, int* __restrict__ row_count, int ncount) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n) out[p] = type[perm[p]];
+  if (p < ncount) row_count[p] = 0;
 }
 
 template <class R>
@@ -927,19 +934,20 @@ int run_fitting(const DeviceModel& m, const PathConst& pc, const R* params, cons
     set_error("scratch allocation failed");
     return DP_E_OOM;
   }
-  for (int t = 0; t < pc.ntypes; ++t) {
-    RowMap rm{0, io.type_start[t], 0, 0, 0, 0, io.type_start[t + 1] - io.type_start[t]};
-    const R* X = D;
-    for (int l = 0; l < nfl; ++l) {
-      const LayerDesc& L = m.fit[(size_t)t * nfl + l];
-      const R* W = params + L.w_off;
-      {
-        ProfScope _ps(io.prof, "fit_fwd", st);
-        DP_CUDA_TRY(launch_dense_fwd<R>(rm, X, L.n_in, W, W + (long)L.n_in * L.n_out, L.n_out, L.skip, L.tanh_act,
-                                        Yf[l], Tf[l], st));
-      }
-      X = Yf[l];
-    }
+  // one launch per layer: the rows of every type with that type's weights
+  auto layer_rows = [&](int l) {
+    DenseRows rows;
+    for (int t = 0; t < pc.ntypes; ++t)
+      rows.add(io.type_start[t], io.type_start[t + 1] - io.type_start[t], m.fit[(size_t)t * nfl + l].w_off);
+    return rows;
+  };
+  auto fit_shape = [](const LayerDesc& L) { return DenseShape{L.n_in, L.n_in, L.n_out, L.n_out, L.skip, L.tanh_act}; };
+  const R* X = D;
+  for (int l = 0; l < nfl; ++l) {
+    const LayerDesc& L = m.fit[l];
+    ProfScope _ps(io.prof, "fit_fwd", st);
+    DP_CUDA_TRY(launch_dense_fwd<R>(layer_rows(l), fit_shape(L), params, X, Yf[l], Tf[l], st));
+    X = Yf[l];
   }
   {
     ProfScope _ps(io.prof, "energy_sum", st);
@@ -950,17 +958,12 @@ int run_fitting(const DeviceModel& m, const PathConst& pc, const R* params, cons
     ProfScope _ps(io.prof, "fill", st);
     k_fill<R><<<nblk(N, 256), 256, 0, st>>>(gA, N, R(1));
   }
-  // layer by layer over all types, so both ping-pong buffers always hold one layer's stride
   R* gy = gA;
   R* gx = gB;
   for (int l = nfl - 1; l >= 0; --l) {
-    for (int t = 0; t < pc.ntypes; ++t) {
-      RowMap rm{0, io.type_start[t], 0, 0, 0, 0, io.type_start[t + 1] - io.type_start[t]};
-      const LayerDesc& L = m.fit[(size_t)t * nfl + l];
-      ProfScope _ps(io.prof, "fit_bwd", st);
-      DP_CUDA_TRY(launch_dense_bwd<R>(rm, gy, L.tanh_act ? Tf[l] : nullptr, L.n_in, params + L.w_off, L.n_out, L.skip,
-                                      gx, st));
-    }
+    const LayerDesc& L = m.fit[l];
+    ProfScope _ps(io.prof, "fit_bwd", st);
+    DP_CUDA_TRY(launch_dense_bwd<R>(layer_rows(l), fit_shape(L), params, gy, Tf[l], gx, st));
     std::swap(gy, gx);
   }
   *gD_out = gy;
@@ -977,6 +980,7 @@ struct PartBufs {
   R* gR = nullptr;         // [rows][4]
   R* gs = nullptr;         // two-body parts: dE/ds through the nets [rows]
   NetPtrs<R> nets;         // first layers of the part's nets
+  RowLists lists;          // two-body parts on layer kernels: the real slot rows per type pair
 };
 
 bool e3_supported(const PartDesc& P, int precision) {
@@ -1217,7 +1221,28 @@ int run_generic(const DeviceModel& m, const PathConst& pc, const R* params, cons
   // se_e2_r parts on the fused per-neighbour kernel (uncompressed nets)
   auto rfused = [&](int q) { return !tabulated(q) && rnet_supported(m.parts[q], m.precision); };
   int* range_flag = &io.status->table_range;
+  // rows of part q's layer l: every (centre type, neighbour type) pair's list with that pair's net
+  auto part_rows = [&](int q, int l) {
+    const PartDesc& P = m.parts[q];
+    DenseRows r;
+    r.list = pb[q].lists.list;
+    r.count = pb[q].lists.count;
+    for (int ti = 0; ti < pc.ntypes; ++ti)
+      for (int tj = 0; tj < pc.ntypes; ++tj) {
+        const int net = pc.type_one_side ? tj : ti * pc.ntypes + tj;
+        r.add(pb[q].lists.base[r.ngroups], (io.type_start[ti + 1] - io.type_start[ti]) * P.sel[tj],
+              P.emb[(size_t)net * P.nl + l].w_off);
+      }
+    return r;
+  };
+  int* row_count = ar.get<int>(nparts * kMaxDenseGroups);
   long maxe = 1;  // widest embedding-gradient buffer over the parts
+  // row stride of layer l's activations: the last layer's rows are read by the descriptor kernels
+  auto emb_ld = [](const PartDesc& P, int l) { return l == P.nl - 1 ? P.emb[l].n_out : dense_ld(P.emb[l].n_out); };
+  auto emb_shape = [&](const PartDesc& P, int l) {
+    const LayerDesc& L = P.emb[l];
+    return DenseShape{L.n_in, emb_ld(P, l - 1), L.n_out, emb_ld(P, l), L.skip, 1};
+  };
   for (int q = 0; q < nparts; ++q) {
     const PartDesc& P = m.parts[q];
     PartBufs<R>& b = pb[q];
@@ -1227,13 +1252,21 @@ int run_generic(const DeviceModel& m, const PathConst& pc, const R* params, cons
     b.gR = ar.get<R>(rows * 4);
     if (P.kind == PART_E3 || tabulated(q) || rfused(q)) continue;
     for (int l = 0; l < P.nl; ++l) {
-      const int w = P.emb[l].n_out;
+      const int w = emb_ld(P, l);
       b.Y.push_back(ar.get<R>(rows * w));
       b.T.push_back(ar.get<R>(rows * w));
       maxe = std::max(maxe, rows * w);
     }
     if (P.kind == PART_A) b.Tm = ar.get<R>(N * P.M * 4);
     b.gs = ar.get<R>(rows);
+    b.lists.list = ar.get<int>(rows);
+    b.lists.count = row_count + q * kMaxDenseGroups;
+    long at = 0;
+    for (int ti = 0; ti < pc.ntypes; ++ti)
+      for (int tj = 0; tj < pc.ntypes; ++tj) {
+        b.lists.base[ti * pc.ntypes + tj] = at;
+        at += (long)(io.type_start[ti + 1] - io.type_start[ti]) * P.sel[tj];
+      }
   }
   R* D = ar.get<R>(N * pc.Dw);
   R* geA = ar.get<R>(maxe);
@@ -1247,7 +1280,8 @@ int run_generic(const DeviceModel& m, const PathConst& pc, const R* params, cons
   }
   {
     ProfScope _ps(io.prof, "sorted_types", st);
-    k_sorted_types<<<nblk(N, 256), 256, 0, st>>>(io.type, io.perm, (int)N, tsorted);
+    k_sorted_types<<<nblk(N, 256), 256, 0, st>>>(io.type, io.perm, (int)N, tsorted, row_count,
+                                                  nparts * kMaxDenseGroups);
   }
   // ---- forward, part by part ----
   for (int q = 0; q < nparts; ++q) {
@@ -1257,7 +1291,7 @@ int run_generic(const DeviceModel& m, const PathConst& pc, const R* params, cons
     const long rows = N * P.nc;
     {
       ProfScope _ps(io.prof, "env", st);
-      k_env<R><<<nblk(rows, 256), 256, 0, st>>>(pq, io.coord, io.perm, io.nl_j, io.nl_code, b.Renv);
+      k_env<R><<<nblk(rows, 256), 256, 0, st>>>(pq, io.coord, io.perm, io.nl_j, io.nl_code, tsorted, b.lists, b.Renv);
     }
     if (P.kind == PART_E3) {
       ProfScope _ps(io.prof, "e3_fwd", st);
@@ -1285,23 +1319,13 @@ int run_generic(const DeviceModel& m, const PathConst& pc, const R* params, cons
     {
       const LayerDesc& L0 = P.emb[0];
       ProfScope _ps(io.prof, "emb_first", st);
-      k_emb_first<R><<<nblk(rows * L0.n_out, 256), 256, 0, st>>>(pq, b.nets, tsorted, b.Renv, L0.n_out, L0.skip,
-                                                                    b.Y[0], b.T[0]);
+      k_emb_first<R><<<nblk(rows * L0.n_out, 256), 256, 0, st>>>(pq, b.nets, tsorted, b.Renv, L0.n_out, emb_ld(P, 0),
+                                                                    L0.skip, b.Y[0], b.T[0]);
     }
-    for (int ti = 0; ti < pc.ntypes; ++ti)
-      for (int tj = 0; tj < pc.ntypes; ++tj) {
-        const int net = pc.type_one_side ? tj : ti * pc.ntypes + tj;
-        RowMap rm{1, 0, io.type_start[ti], pq.sel[tj], pq.sel_off[tj], P.nc,
-                  (io.type_start[ti + 1] - io.type_start[ti]) * pq.sel[tj]};
-        rm.zrow = b.Renv;  // padding rows: no layer outputs
-        for (int l = 1; l < P.nl; ++l) {
-          const LayerDesc& L = P.emb[(size_t)net * P.nl + l];
-          const R* W = params + L.w_off;
-          ProfScope _ps(io.prof, "emb_fwd", st);
-          DP_CUDA_TRY(launch_dense_fwd<R>(rm, b.Y[l - 1], L.n_in, W, W + (long)L.n_in * L.n_out, L.n_out, L.skip, 1,
-                                          b.Y[l], b.T[l], st));
-        }
-      }
+    for (int l = 1; l < P.nl; ++l) {  // padding rows are in no list: no layer outputs for them
+      ProfScope _ps(io.prof, "emb_fwd", st);
+      DP_CUDA_TRY(launch_dense_fwd<R>(part_rows(q, l), emb_shape(P, l), params, b.Y[l - 1], b.Y[l], b.T[l], st));
+    }
     const R* G = b.Y[P.nl - 1];
     if (P.kind == PART_A) {
       ProfScope _ps(io.prof, "contract", st);
@@ -1344,22 +1368,14 @@ int run_generic(const DeviceModel& m, const PathConst& pc, const R* params, cons
       R* gy = geA;
       R* gx = geB;
       for (int l = P.nl - 1; l >= 1; --l) {
-        for (int ti = 0; ti < pc.ntypes; ++ti)
-          for (int tj = 0; tj < pc.ntypes; ++tj) {
-            const int net = pc.type_one_side ? tj : ti * pc.ntypes + tj;
-            RowMap rm{1, 0, io.type_start[ti], pq.sel[tj], pq.sel_off[tj], P.nc,
-                      (io.type_start[ti + 1] - io.type_start[ti]) * pq.sel[tj]};
-            rm.zrow = b.Renv;
-            const LayerDesc& L = P.emb[(size_t)net * P.nl + l];
-            ProfScope _ps(io.prof, "emb_bwd", st);
-            DP_CUDA_TRY(launch_dense_bwd<R>(rm, gy, b.T[l], L.n_in, params + L.w_off, L.n_out, L.skip, gx, st));
-          }
+        ProfScope _ps(io.prof, "emb_bwd", st);
+        DP_CUDA_TRY(launch_dense_bwd<R>(part_rows(q, l), emb_shape(P, l), params, gy, b.T[l], gx, st));
         std::swap(gy, gx);
       }
       const LayerDesc& L0 = P.emb[0];
       ProfScope _ps(io.prof, "emb_first_bwd", st);
-      k_emb_first_bwd<R><<<nblk(rows, 256), 256, 0, st>>>(pq, b.nets, tsorted, b.Renv, gy, b.T[0], L0.n_out, L0.skip,
-                                                         b.gs);
+      k_emb_first_bwd<R><<<nblk(rows, 256), 256, 0, st>>>(pq, b.nets, tsorted, b.Renv, gy, b.T[0], L0.n_out,
+                                                         emb_ld(P, 0), L0.skip, b.gs);
     }
     ProfScope _ps(io.prof, "force", st);
     k_force<R><<<nblk(rows, 256), 256, 0, st>>>(pq, io.coord, io.perm, io.nl_j, io.nl_code, b.gs, b.gR, io.force,
