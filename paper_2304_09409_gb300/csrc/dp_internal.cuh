@@ -215,8 +215,10 @@ inline cudaError_t allow_max_smem(K kernel) {
 // ------------------------------------------------------------------------------------------
 // Launchers (nlist.cu)
 // ------------------------------------------------------------------------------------------
+// Cell grid of one frame.  fine: cells narrower than r_c are allowed where they save candidates (not for
+// callers that keep the list's FP32 displacements, whose rounding follows the grid).
 int host_geometry(const dp_model_config& cfg, int natoms, const double* box_host, const double* bbox_lohi,
-                  NlGeom& g);
+                  NlGeom& g, bool fine = false);
 cudaError_t launch_bbox(const double* coord, int natoms, double* out_lohi /*device [6]*/, cudaStream_t st);
 // One neighbour-list build over one or more frames of the same model.
 struct NlLaunch {
@@ -229,6 +231,7 @@ struct NlLaunch {
   int nframes;            // frames in the launch
   int max_noff;           // largest (2K_0+1)(2K_1+1)(2K_2+1) over the frames
   int max_stream;         // largest mean candidate stream of one cell over the frames (0: unknown)
+  double max_cell_atoms = 0.0;  // largest mean number of atoms of a cell over the frames (0: unknown)
 };
 // What a path call also takes from the list build: the (type, cell) order of the atoms as its
 // type-sorted order (perm [natoms], type_start [ntypes + 1], checked against chk) and the 27
@@ -245,6 +248,10 @@ struct NlExtras {
   // decided, -1 for padding; written only by the cell-centred search (disp_written says so)
   float4* disp;
   bool disp_written;
+  // the list's readers walk each type block in 32-slot batches and stop at the first batch with padding:
+  // padding beyond that batch may stay unwritten
+  bool lean;
+  bool counts_clear;  // cell_count is zero already
 };
 // Cell arrays are indexed by (type, cell): cell_count [ntypes * ncells_total], cell_start
 // [ntypes * ncells_total + 1]; per atom its key and rank within the key (atom_key, int2), its

@@ -46,35 +46,27 @@ __global__ void k_shift_tables(const double* __restrict__ boxes, double* __restr
 }
 
 // Per-chunk sums of atom energies and atom virials (10 values), fixed order; the block that
-// finishes a frame's last chunk then forms the frame's sums from the chunk partials, thread k
-// adding chunks k, k + 128, ... of the frame and a fixed tree over the threads (the order depends
-// on the frame alone, not on the batch or on which block finished last).  fcount[f] counts the
+// finishes a frame's last chunk then forms the frame's sums from the chunk partials in the same way
+// (the order depends on the frame alone, not on the batch or on which block finished last).  fcount[f] counts the
 // finished chunks of frame f; it is zero on entry and left zero.
-__global__ void __launch_bounds__(kChunk)
+// A warp per component: four values a lane and a shuffle tree, i.e. nine dependent additions a stage on
+// the FP64 pipe (about two additions a clock and SM); what is left is the chain of memory round trips.
+__global__ void __launch_bounds__(320)
     k_chunk_sums(const int* __restrict__ chunk, const double* __restrict__ ae, const double* __restrict__ av,
                  double* __restrict__ cpart, const int* __restrict__ frame_chunk, int nframes, int* __restrict__ fcount,
                  double* __restrict__ energy, double* __restrict__ virial) {
-  static_assert(kChunk == 128, "four warps per chunk block");
-  __shared__ double red[4][10];
   __shared__ int s_last;
-  const int c = blockIdx.x;
-  const int beg = chunk[2 * c], end = chunk[2 * c + 1];
-  double acc[10];
+  const int c = blockIdx.x, lane = threadIdx.x & 31, q = threadIdx.x >> 5;  // component q
+  // the sum over n rows of one component, rows s apart
+  auto sum_rows = [&](const double* v, long s, int n) {
+    double x = 0.0;
+#pragma unroll 4
+    for (int r = lane; r < n; r += 32) x += __ldcg(v + r * s);
 #pragma unroll
-  for (int q = 0; q < 10; ++q) acc[q] = 0.0;
-  for (int i = beg + threadIdx.x; i < end; i += blockDim.x) {
-    acc[0] += ae[i];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) acc[1 + q] += av[9L * i + q];
-  }
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < 10; ++q) {
-    double x = acc[q];
     for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-    if (lane == 0) red[w][q] = x;
-  }
-  __syncthreads();
+    return x;
+  };
+  const int beg = chunk[2 * c], end = chunk[2 * c + 1];
   int f = 0;  // frame of this chunk
   {
     int lo = 0, hi = nframes - 1;
@@ -85,10 +77,14 @@ __global__ void __launch_bounds__(kChunk)
     f = lo;
   }
   const int c0 = frame_chunk[f], c1 = frame_chunk[f + 1];
-  if (threadIdx.x < 10) {
-    double x = 0.0;
-    for (int k = 0; k < 4; ++k) x += red[k][threadIdx.x];
-    cpart[10L * c + threadIdx.x] = x;
+  const double part = q == 0 ? sum_rows(ae + beg, 1, end - beg) : sum_rows(av + 9L * beg + q - 1, 9, end - beg);
+  double* out = q == 0 ? energy + f : virial + 9L * f + q - 1;
+  if (c1 - c0 == 1) {  // the frame's only chunk
+    if (lane == 0) *out = part;
+    return;
+  }
+  if (lane == 0) {
+    __stcg(cpart + 10L * c + q, part);
     __threadfence();
   }
   __syncthreads();
@@ -96,27 +92,22 @@ __global__ void __launch_bounds__(kChunk)
   __syncthreads();
   if (!s_last) return;  // block-uniform
   __threadfence();
-  const int tid = threadIdx.x;
+  const double x = sum_rows(cpart + 10L * c0 + q, 10, c1 - c0);
+  if (lane == 0) *out = x;
+  if (threadIdx.x == 0) fcount[f] = 0;
+}
+
+// Everything a call starts from zero, in one launch (each memset was a node of its own in the call's
+// graph, and the only nodes that touched the caller's buffers other than by a kernel).
+struct ClearArgs {
+  unsigned* p[5];
+  long n[5];  // 32-bit words
+};
+__global__ void k_clear(const ClearArgs a) {
+  const long t = (long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long)gridDim.x * blockDim.x;
 #pragma unroll
-  for (int q = 0; q < 10; ++q) acc[q] = 0.0;
-  for (int cc = c0 + tid; cc < c1; cc += kChunk)
-#pragma unroll
-    for (int q = 0; q < 10; ++q) acc[q] += __ldcg(cpart + 10L * cc + q);
-#pragma unroll
-  for (int q = 0; q < 10; ++q) {
-    double x = acc[q];
-    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-    if (lane == 0) red[w][q] = x;
-  }
-  __syncthreads();
-  if (tid < 10) {
-    const double x = (red[0][tid] + red[1][tid]) + (red[2][tid] + red[3][tid]);
-    if (tid == 0)
-      energy[f] = x;
-    else
-      virial[9L * f + tid - 1] = x;
-  }
-  if (tid == 0) fcount[f] = 0;
+  for (int k = 0; k < 5; ++k)
+    for (long e = t; e < a.n[k]; e += nt) a.p[k][e] = 0u;
 }
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -162,6 +153,12 @@ struct FrameTables {
     }
     return (int)std::ceil(m);
   }
+  double max_cell_atoms() const {
+    double m = 0.0;
+    for (int f = 0; f < F; ++f)
+      m = std::max(m, (double)(start[f + 1] - start[f]) / std::max(1, cell_off[f + 1] - cell_off[f]));
+    return m;
+  }
   void pack(unsigned char* p) const {
     std::memcpy(p + off_geoms, geoms.data(), sizeof(NlGeom) * F);
     std::memcpy(p + off_celloff, cell_off.data(), sizeof(int) * (F + 1));
@@ -190,7 +187,8 @@ int build_tables_host(dp_model* md, int F, const int* natoms, const double* boxe
   T.boxes.assign(9 * (size_t)F, 0.0);
   T.cap = 0;
   for (int f = 0; f < F; ++f) {
-    const int rc = host_geometry(md->m.lcfg, natoms[f], boxes ? boxes + 9 * f : nullptr, lohi, T.geoms[f]);
+    const int rc = host_geometry(md->m.lcfg, natoms[f], boxes ? boxes + 9 * f : nullptr, lohi, T.geoms[f],
+                                  !(md->m.compressed && md->m.mom_npass == 1));
     if (rc != DP_OK) return rc;
     NlGeom& g = T.geoms[f];
     if (md->nl_full_cap) g.cap = DP_MAX_CANDIDATES;
@@ -430,7 +428,26 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
     const int* d_chunk = reinterpret_cast<const int*>(b.ftab + T.off_chunk);
     const int* d_fchunk = reinterpret_cast<const int*>(b.ftab + T.off_fchunk);
     const double* d_boxes = reinterpret_cast<const double*>(b.ftab + T.off_boxes);
-    DP_CUDA_TRY(cudaMemsetAsync(md->status, 0, sizeof(DevStatus), s));
+    {
+      ClearArgs ca;
+      std::memset(&ca, 0, sizeof(ca));
+      int k = 0;
+      long most = 0;
+      auto clear = [&](void* p, size_t bytes) {
+        ca.p[k] = reinterpret_cast<unsigned*>(p);
+        ca.n[k] = (long)(bytes / 4);
+        most = std::max(most, ca.n[k++]);
+      };
+      clear(md->status, sizeof(DevStatus));
+      if (own_nlist) clear(b.cell_count, sizeof(int) * (size_t)T.ncells * m.cfg.ntypes);
+      if (!gr) {
+        clear(host_f ? b.force : force, sizeof(double) * 3 * N);
+        clear(b.fcount, sizeof(int) * F);
+        if (!m.compressed) clear(b.atom_virial, sizeof(double) * 9 * N);
+      }
+      ProfScope _ps(&md->prof, "clear", s);
+      k_clear<<<(unsigned)std::min<long>((most + 255) / 256, 4L * sm_count()), 256, 0, s>>>(ca);
+    }
     if (F > 1) {
       ProfScope _ps(&md->prof, "atom_frame", s);
       k_atom_frame<<<(N + 255) / 256, 256, 0, s>>>(d_start, F, N, b.atom_frame);
@@ -439,9 +456,11 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
       // the list build's (type, cell) order is the path's type-sorted order, and its first
       // launch also forms the image translations
       NlLaunch L{N, T.ncells, T.cap, d_geoms, b.atom_frame, F > 1 ? d_celloff : nullptr, F, T.max_noff(),
-                 T.max_stream()};
+                 T.max_stream(), T.max_cell_atoms()};
+      // the moment path reads its list in batches
+      const bool lean = m.compressed && m.cfg.descriptor == DP_DESC_SE_E2_A && m.mom_npass != 0;
       NlExtras ex{b.perm, b.type_start, chk, d_boxes, T.periodic ? F : 0, T.periodic ? b.tshift : nullptr, b.disp,
-                  false};
+                  false, lean, true};
       ProfScope _ps(&md->prof, "nlist", s, nlist_launches(L, m.cfg.ntypes));
       const NlScratch sc{b.cell_count, b.cell_start, b.atom_key, b.atom_l, b.atom_m, b.sorted_l, b.sorted_m};
       DP_CUDA_TRY(launch_nlist_build(L, m.cfg.ntypes, dcoord, dtype, sc, b.nl_j, b.nl_code, b.counts, md->status, s,
@@ -494,16 +513,13 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
         DP_CUDA_TRY(cudaMemcpyAsync(gr->grad, d_gout, sizeof(double) * m.n_params, cudaMemcpyDeviceToHost, s));
       return DP_OK;
     }
-    DP_CUDA_TRY(cudaMemsetAsync(io.force, 0, sizeof(double) * 3 * N, s));
-    DP_CUDA_TRY(cudaMemsetAsync(b.fcount, 0, sizeof(int) * F, s));
-    if (!m.compressed) DP_CUDA_TRY(cudaMemsetAsync(io.atom_virial, 0, sizeof(double) * 9 * N, s));
     int r = run_path(m, pc, io, ar, s);
     if (r != DP_OK) return r;
     double* d_energy = host_e ? b.energy : energy;
     double* d_virial = host_v ? b.virial : virial;
     {
       ProfScope _ps(&md->prof, "frame_sums", s);
-      k_chunk_sums<<<T.C, kChunk, 0, s>>>(d_chunk, io.atom_energy, io.atom_virial, b.cpart, d_fchunk, F, b.fcount,
+      k_chunk_sums<<<T.C, 320, 0, s>>>(d_chunk, io.atom_energy, io.atom_virial, b.cpart, d_fchunk, F, b.fcount,
                                           d_energy, d_virial);
     }
     DP_CUDA_TRY(cudaGetLastError());
@@ -756,7 +772,7 @@ int dp_build_nlist(dp_model* md, int N, const double* coord, const int* type, co
   DP_CUDA_TRY(cudaMemsetAsync(md->status, 0, sizeof(DevStatus), st));
   {
     NlLaunch L{N, T.ncells, T.cap, reinterpret_cast<const NlGeom*>(b.ftab + T.off_geoms), nullptr, nullptr, 1,
-               T.max_noff(), T.max_stream()};
+               T.max_noff(), T.max_stream(), T.max_cell_atoms()};
     ProfScope _ps(&md->prof, "nlist", st, nlist_launches(L, m.cfg.ntypes));
     const NlScratch sc{b.cell_count, b.cell_start, b.atom_key, b.atom_l, b.atom_m, b.sorted_l, b.sorted_m};
     DP_CUDA_TRY(launch_nlist_build(L, m.cfg.ntypes, dcoord, dtype, sc, nl->nl_j, nl->nl_code, nl->counts, md->status,

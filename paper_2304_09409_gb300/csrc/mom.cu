@@ -1135,9 +1135,11 @@ __global__ void __launch_bounds__(256)
   while (t < pc.ntypes) {
     const int kb0 = g.sel_off[t], kb1 = g.sel_off[t + 1];
     const int jc = jn;
-    const bool any = __any_sync(0xffffffffu, jc >= 0);  // real neighbours fill the front of the block
+    // real neighbours fill the front of the block: a batch that is not full ends it (a lean list holds
+    // nothing behind that batch)
+    const bool full = __all_sync(0xffffffffu, jc >= 0);
     int tn = t, bn = base + 32;
-    if (!any || bn >= kb1) {
+    if (!full || bn >= kb1) {
       tn = t + 1;
       bn = tn < pc.ntypes ? g.sel_off[tn] : 0;
     }
@@ -1147,7 +1149,6 @@ __global__ void __launch_bounds__(256)
     t = tn;
     base = bn;
     {
-      if (!any) continue;
       const int j = jc;
       if (j < 0) continue;
       const long row = (long)p * pc.nc + k;

@@ -170,39 +170,37 @@ __global__ void k_scan_excl(const int* __restrict__ in, int n, int* __restrict__
 }
 
 // Exclusive scan of the key counts into shared memory by one block (a few thousand keys: every
-// block of the fill forms it itself instead of waiting for a separate scan launch).
+// block of the fill forms it itself instead of waiting for a separate scan launch): each thread takes
+// a contiguous stretch, so that one round of the warp scan serves any number of keys.
 __device__ __forceinline__ void block_scan_counts(const int* __restrict__ in, int n, int* s_out) {
   __shared__ int wsum[32];
-  __shared__ int carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-  for (int base = 0; base < n; base += blockDim.x) {
-    const int idx = base + threadIdx.x;
-    const int v = idx < n ? in[idx] : 0;
-    int incl = v;
-    for (int off = 1; off < 32; off <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += t;
-    }
-    if (lane == 31) wsum[w] = incl;
-    __syncthreads();
-    if (w == 0) {
-      int x = lane < nw ? wsum[lane] : 0;
-      for (int off = 1; off < 32; off <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, x, off);
-        if (lane >= off) x += t;
-      }
-      wsum[lane] = x;
-    }
-    __syncthreads();
-    const int before = (w > 0 ? wsum[w - 1] : 0) + carry;
-    if (idx < n) s_out[idx] = before + incl - v;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry = before + incl;
-    __syncthreads();
+  for (int k = threadIdx.x; k < n; k += blockDim.x) s_out[k] = in[k];
+  __syncthreads();
+  const int per = (n + (int)blockDim.x - 1) / (int)blockDim.x | 1;  // odd: no bank conflicts
+  const int k0 = min(n, (int)threadIdx.x * per), k1 = min(n, k0 + per);
+  int sum = 0;
+  for (int k = k0; k < k1; ++k) sum += s_out[k];
+  int incl = sum;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += t;
   }
-  if (threadIdx.x == 0) s_out[n] = carry;
+  if (lane == 31) wsum[w] = incl;
+  __syncthreads();
+  int run = incl - sum;
+  for (int k = 0; k < w; ++k) run += wsum[k];
+  for (int k = k0; k < k1; ++k) {
+    const int v = s_out[k];
+    s_out[k] = run;
+    run += v;
+  }
+  if (threadIdx.x == blockDim.x - 1) {
+    int total = 0;
+    for (int k = 0; k < nw; ++k) total += wsum[k];
+    s_out[n] = total;
+  }
   __syncthreads();
 }
 
@@ -552,12 +550,19 @@ __global__ void __launch_bounds__(kNlWarps * 32)
 constexpr int kCellWarps = 8;
 constexpr int kMaxRanges = 256;  // (type, surrounding cell) ranges of one cell
 
-// Dynamic shared memory: S staged candidates (24 bytes each) and per warp an entry buffer of
-// cap + 4 entries (FP32 key, 16-bit stream position, 16-bit entry index in bucket order) and
-// cap bucket counters (the FP32 keys of one type group are bucketed over [0, r_c^2 + eps], as
-// many buckets as the buffer has entries).
+// Key buckets per warp: the FP32 keys of one type group are bucketed over [0, r_c^2 + eps].  Half the
+// buffer's entries (twice the mean group) is about one entry a bucket.
+__host__ __device__ constexpr int cell_buckets(int cap) { return cap <= 256 ? 128 : 256; }
+
+// Dynamic shared memory: S staged candidates (24 bytes each) and per warp an entry buffer of cap + 8
+// entries (FP32 key and 16-bit stream position) and 16-bit bucket counters.  The buffer is put into
+// bucket order in place, through registers: with a second buffer two blocks fitted an SM on the metal
+// crystal (r_c 8, 448 entries) instead of three.
+__host__ __device__ constexpr size_t cell_warp_bytes(int cap) {
+  return (size_t)(cap + 8) * 6 + (size_t)cell_buckets(cap) * 2;
+}
 __host__ __device__ constexpr size_t cell_smem_bytes(int cap, int S) {
-  return (size_t)S * 24 + (size_t)kCellWarps * ((size_t)(cap + 4) * 8 + (size_t)cap * 4);
+  return (size_t)S * 24 + (size_t)kCellWarps * cell_warp_bytes(cap);
 }
 
 // Bucket of an FP32 key: monotone in x, so that every key of a lower bucket is smaller and every
@@ -627,14 +632,14 @@ __device__ __forceinline__ bool staged_code(unsigned long long wm, int mi0, int 
 }
 
 template <int CAP>
-__global__ void __launch_bounds__(kCellWarps * 32, 4)
+__global__ void __launch_bounds__(kCellWarps * 32, CAP <= 256 ? 4 : 3)
     k_nlist_cell(const NlGeom* __restrict__ G, const int* __restrict__ cell_off, int nframes, int ncells_total,
                  int ntypes, const double* __restrict__ coord, const int* __restrict__ cell_start,
                  const float4* __restrict__ sorted_l, const int4* __restrict__ sorted_m, int S, int* __restrict__ nl_j,
-                 int* __restrict__ nl_code, int* __restrict__ counts, float4* __restrict__ disp,
-                 DevStatus* __restrict__ st) {
+                 int* __restrict__ nl_code, int* __restrict__ counts, float4* __restrict__ disp, int per_block,
+                 bool lean, DevStatus* __restrict__ st) {
   constexpr int NT = kCellWarps * 32;
-  constexpr int CAPP = CAP + 4;
+  constexpr int CAPP = CAP + 8;
   extern __shared__ __align__(16) unsigned char smem[];
   float4* stg = reinterpret_cast<float4*>(smem);                                        // l_j + o, j
   unsigned long long* stg_w = reinterpret_cast<unsigned long long*>(smem + (size_t)S * 16);  // W - m_j
@@ -644,13 +649,24 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4)
   __shared__ int s_sel[DP_MAX_TYPES], s_seloff[DP_MAX_TYPES];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
-  constexpr int NB = CAP;  // key buckets
-  float* e_key = reinterpret_cast<float*>(smem + (size_t)S * 24 + (size_t)warp * (CAPP * 8 + NB * 4));
-  unsigned short* e_ref = reinterpret_cast<unsigned short*>(e_key + CAPP);  // stream position (S < 2^16)
-  unsigned short* e_idx = e_ref + CAPP;                                     // entries in bucket order
-  int* e_hist = reinterpret_cast<int*>(e_idx + CAPP);                       // bucket ends
+  constexpr int NB = cell_buckets(CAP);
+  // entries, as accepted and later in bucket order: FP32 key, stream position (S < 2^16)
+  float* e_key = reinterpret_cast<float*>(smem + (size_t)S * 24 + (size_t)warp * cell_warp_bytes(CAP));
+  unsigned* hist = reinterpret_cast<unsigned*>(e_key + CAPP);  // two 16-bit counters a word; then bucket ends
+  unsigned short* e_ref = reinterpret_cast<unsigned short*>(hist + NB / 2);
 
   const int gc = blockIdx.x;  // cell, all frames
+  // this block's share of the cell's centre atoms: per_block of them from blockIdx.y * per_block on
+  // (and again every gridDim.y * per_block where the cell holds more than expected)
+  const int first = (int)blockIdx.y * per_block;
+  {
+    int n = 0;
+    for (int t = 0; t < ntypes; ++t) {
+      const int key = t * ncells_total + gc;
+      n += __ldg(cell_start + key + 1) - __ldg(cell_start + key);
+    }
+    if (n <= first) return;  // CTA-uniform
+  }
   int fr = 0;
   if (cell_off) {  // frame holding this cell
     int lo = 0, hi = nframes - 1;
@@ -738,12 +754,11 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4)
   if (tid < R) s_rpex[tid] += s_tdel[tid / noff];
   const int P = s_tpex[ntypes];
   const int nce = s_cpre[ntypes];
-  if (nce == 0) return;  // CTA-uniform: no centre atom in this cell
   if (P > S) {  // CTA-uniform: the stream does not fit the staging buffer.  The call reports it
                 // (and is retried on the per-atom kernel); meanwhile this cell's rows are left
                 // empty, so that the kernels after the list stay in bounds.
     if (tid == 0) atomicExch(&st->capacity, 1);
-    for (int q = warp; q < nce; q += kCellWarps) {
+    for (int q = warp; q < nce && blockIdx.y == 0; q += kCellWarps) {
       int tc = 0;
       while (tc + 1 < ntypes && s_cpre[tc + 1] <= q) ++tc;
       const int w = s_rbeg[tc * noff + oc] + q - s_cpre[tc];
@@ -789,7 +804,8 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4)
   const int nc = g.nc;
   const unsigned lt = (1u << lane) - 1u;
   const float kInf = __int_as_float(0x7f800000);
-  for (int q = warp; q < nce; q += kCellWarps) {
+  const int stride = (int)gridDim.y * per_block;
+  for (int q = first + warp; q < nce;) {
     int tc = 0;
     while (tc + 1 < ntypes && s_cpre[tc + 1] <= q) ++tc;
     const int pc = s_rpex[tc * noff + oc] + q - s_cpre[tc];  // the centre's own entry (W = 0)
@@ -839,13 +855,13 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4)
       const int ge = min(cnt, CAP);
       __syncwarp();
       // ---- bucket order of the surviving FP32 keys ----
-      // Counting sort into NB buckets of the keys' range: counts, exclusive scan, scatter of the
-      // entry indices; afterwards e_hist[b] is the end of bucket b in e_idx.  The counting pass
-      // first settles the entries within the FP32 error of r_c by the exact FP64 test (dropped
-      // entries get the key +inf and no bucket).
-      for (int b = lane; b < NB; b += 32) e_hist[b] = 0;
+      // Counting sort into NB buckets of the keys' range, in place: counts, exclusive scan, scatter of keys
+      // and stream positions through registers; afterwards bucket b ends at end_of(b).  The counting pass first settles the entries within the FP32 error of r_c by the
+      // exact FP64 test (dropped entries get the key +inf and no bucket).
+      for (int b = lane; b < NB / 2; b += 32) hist[b] = 0;
       __syncwarp();
       int removed = 0;
+#pragma unroll 1
       for (int e0 = 0; e0 < ge; e0 += 32) {
         const int e = e0 + lane;
         float k = e < ge ? e_key[e] : kInf;
@@ -866,79 +882,92 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4)
           }
           removed += __popc(__ballot_sync(0xffffffffu, drop));
         }
-        if (k != kInf) atomicAdd(&e_hist[key_bucket<NB>(k, inv_bw)], 1);
+        if (k != kInf) {
+          const int b = key_bucket<NB>(k, inv_bw);
+          atomicAdd(&hist[b >> 1], 1u << ((b & 1) << 4));
+        }
       }
       __syncwarp();
       {
-        constexpr int PER = NB / 32;  // buckets per lane, contiguous
-        int c[PER];
-        int sum = 0;
+        constexpr int WPL = NB / 64;  // counter words per lane, contiguous
+        unsigned c[WPL];
+        unsigned sum = 0;
 #pragma unroll
-        for (int v = 0; v < PER / 4; ++v) {
-          const int4 x = reinterpret_cast<const int4*>(e_hist)[lane * (PER / 4) + v];
-          c[4 * v] = x.x;
-          c[4 * v + 1] = x.y;
-          c[4 * v + 2] = x.z;
-          c[4 * v + 3] = x.w;
-          sum += x.x + x.y + x.z + x.w;
+        for (int v = 0; v < WPL; ++v) {
+          c[v] = hist[lane * WPL + v];
+          sum += (c[v] & 0xffffu) + (c[v] >> 16);
         }
-        int incl = sum;
+        unsigned incl = sum;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
-          const int x = __shfl_up_sync(0xffffffffu, incl, off);
+          const unsigned x = __shfl_up_sync(0xffffffffu, incl, off);
           if (lane >= off) incl += x;
         }
-        int run = incl - sum;
+        unsigned run = incl - sum;
 #pragma unroll
-        for (int v = 0; v < PER / 4; ++v) {
-          int4 x;
-          x.x = run;
-          run += c[4 * v];
-          x.y = run;
-          run += c[4 * v + 1];
-          x.z = run;
-          run += c[4 * v + 2];
-          x.w = run;
-          run += c[4 * v + 3];
-          reinterpret_cast<int4*>(e_hist)[lane * (PER / 4) + v] = x;
+        for (int v = 0; v < WPL; ++v) {
+          const unsigned lo = c[v] & 0xffffu;
+          hist[lane * WPL + v] = run | ((run + lo) << 16);
+          run += lo + (c[v] >> 16);
         }
       }
       __syncwarp();
-      for (int e = lane; e < ge; e += 32) {
-        const float k = e_key[e];
-        if (k != kInf) e_idx[atomicAdd(&e_hist[key_bucket<NB>(k, inv_bw)], 1)] = (unsigned short)e;
+      {
+        constexpr int EPL = CAP / 32;
+        float kk[EPL];
+        unsigned rr[EPL];
+#pragma unroll
+        for (int v = 0; v < EPL; ++v) {
+          const int e = 32 * v + lane;
+          kk[v] = e < ge ? e_key[e] : kInf;
+          rr[v] = e < ge ? e_ref[e] : 0;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int v = 0; v < EPL; ++v) {
+          if (32 * v >= ge) break;  // warp-uniform
+          if (kk[v] != kInf) {
+            const int b = key_bucket<NB>(kk[v], inv_bw), sh = (b & 1) << 4;
+            const int pos = (int)((atomicAdd(&hist[b >> 1], 1u << sh) >> sh) & 0xffffu);
+            e_key[pos] = kk[v];
+            e_ref[pos] = (unsigned short)rr[v];
+          }
+        }
       }
       __syncwarp();
+      auto end_of = [&](int b) { return (int)((hist[b >> 1] >> ((b & 1) << 4)) & 0xffffu); };
       // ---- rank under the exact total order (r^2, j, image code) ----
-      // Entries more than the tie window below an entry's key are certainly smaller: all of the
-      // buckets below the window's lower edge and the smaller keys of the edge bucket.  Entries
-      // inside the window (in bucket order between the two edge buckets) take exact keys.
+      // Entries are taken in bucket order, so that the slots a warp writes lie close together.  Entries
+      // more than the tie window below an entry's key are certainly smaller: all of the buckets below
+      // the window's lower edge and the smaller keys of the edge bucket.  Entries inside the window
+      // (in bucket order between the two edge buckets) take exact keys.
       const int sel = s_sel[tj];
       const long row = (long)i * nc + s_seloff[tj];
-      for (int e0 = 0; e0 < ge; e0 += 32) {
+      const int nreal = ge - removed;
+      for (int e0 = 0; e0 < nreal; e0 += 32) {
         const int e = e0 + lane;
-        const float ke = e < ge ? e_key[e] : kInf;
-        const bool valid = ke != kInf;
+        const bool valid = e < nreal;
+        const float ke = valid ? e_key[e] : kInf;
         const float lo_t = ke - tw, hi_t = ke + tw;
         int lo = 0, nle = 0;  // keys certainly smaller; keys not certainly larger
         int wa = 0, wb = 0;   // bucket-order positions spanning the window
         if (valid) {
           const int bl = key_bucket<NB>(lo_t, inv_bw), bh = key_bucket<NB>(hi_t, inv_bw);
-          wa = bl ? e_hist[bl - 1] : 0;
-          wb = e_hist[bh];
+          wa = bl ? end_of(bl - 1) : 0;
+          wb = end_of(bh);
           lo = wa;
           if (bl == bh) {  // the usual case: the window inside one bucket
             nle = wa;
             for (int q = wa; q < wb; ++q) {
-              const float kq = e_key[e_idx[q]];
+              const float kq = e_key[q];
               lo += kq < lo_t;
               nle += kq <= hi_t;
             }
           } else {
-            for (int q = wa, qe = e_hist[bl]; q < qe; ++q) lo += e_key[e_idx[q]] < lo_t;
-            const int sh = e_hist[bh - 1];
+            for (int q = wa, qe = end_of(bl); q < qe; ++q) lo += e_key[q] < lo_t;
+            const int sh = end_of(bh - 1);
             nle = sh;
-            for (int q = sh; q < wb; ++q) nle += e_key[e_idx[q]] <= hi_t;
+            for (int q = sh; q < wb; ++q) nle += e_key[q] <= hi_t;
           }
         }
         int je = 0, ce = 0;
@@ -962,8 +991,7 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4)
             const int wa_s = __shfl_sync(0xffffffffu, wa, s), wb_s = __shfl_sync(0xffffffffu, wb, s);
             int add = 0;
             for (int q0 = wa_s; q0 < wb_s; q0 += 32) {
-              const int q = q0 + lane;
-              const int f = q < wb_s ? e_idx[q] : -1;
+              const int f = q0 + lane < wb_s ? q0 + lane : -1;
               const float kf = f >= 0 ? e_key[f] : kInf;
               const bool in = f >= 0 && f != e0 + s && kf >= lo_s && kf <= hi_s;
               // a partner that is an ambiguous entry of this pass has its exact key in its lane
@@ -1007,11 +1035,10 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4)
       // ---- padding, counts and overflow accounting of this type ----
       // The displacements' reader walks a type block in 32-slot batches and stops after the first
       // batch that holds padding, so padding displacements are written only up to the end of the
-      // batch after the last real neighbour.
+      // batch after the last real neighbour; a lean list's other rows as well (its readers stop there).
       const int ng = cnt - removed;  // entries beyond CAP (an error) are not in the list
-      const int nreal = ge - removed;
       const int dlim = min(sel, ((nreal >> 5) + 1) << 5);
-      for (int k = nreal + lane; k < sel; k += 32) {
+      for (int k = nreal + lane; k < (lean ? dlim : sel); k += 32) {
         nl_j[row + k] = -1;
         nl_code[row + k] = pack_shift(0, 0, 0);
         if (disp && k < dlim) disp[(long)w * nc + s_seloff[tj] + k] = make_float4(0.f, 0.f, 0.f, -1.f);
@@ -1024,6 +1051,9 @@ __global__ void __launch_bounds__(kCellWarps * 32, 4)
     }
     if (__any_sync(0xffffffffu, bad_shift) && lane == 0) atomicExch(&st->capacity, 2);
     if (over && lane == 0) atomicExch(&st->capacity, 1);
+    // the block's next centre atom: 8 further on, or in its next share
+    const int nq = q + kCellWarps;
+    q = (nq - first) % stride < per_block ? nq : nq - (nq - first) % stride + stride + warp;
   }
 }
 
@@ -1160,7 +1190,8 @@ int screening_bounds(NlGeom& g, double rc) {
 
 }  // namespace
 
-int host_geometry(const dp_model_config& cfg, int natoms, const double* box, const double* lohi, NlGeom& g) {
+int host_geometry(const dp_model_config& cfg, int natoms, const double* box, const double* lohi, NlGeom& g,
+                  bool fine) {
   std::memset(&g, 0, sizeof(g));
   g.natoms = natoms;
   g.ntypes = cfg.ntypes;
@@ -1189,25 +1220,47 @@ int host_geometry(const dp_model_config& cfg, int natoms, const double* box, con
     g.inv[3] = c01 / det; g.inv[4] = (h[0] * h[8] - h[2] * h[6]) / det; g.inv[5] = (h[2] * h[3] - h[0] * h[5]) / det;
     g.inv[6] = c02 / det; g.inv[7] = (h[1] * h[6] - h[0] * h[7]) / det; g.inv[8] = (h[0] * h[4] - h[1] * h[3]) / det;
     const double vol = std::fabs(det);
-    long total = 1;
+    double width[3];
     for (int d = 0; d < 3; ++d) {
       const double* u = h + 3 * ((d + 1) % 3);
       const double* v = h + 3 * ((d + 2) % 3);
       double cx = u[1] * v[2] - u[2] * v[1], cy = u[2] * v[0] - u[0] * v[2], cz = u[0] * v[1] - u[1] * v[0];
-      double width = vol / std::sqrt(cx * cx + cy * cy + cz * cz);
-      int n = (int)std::floor(width / cellmin);
-      if (n < 1) n = 1;
-      if (n > 256) n = 256;
-      g.ncell[d] = n;
-      g.K[d] = (int)std::ceil(cellmin * n / width);
-      if (g.K[d] < 1) g.K[d] = 1;
+      width[d] = vol / std::sqrt(cx * cx + cy * cy + cz * cz);
+    }
+    // cells of at least r_c / div; returns the part of the box's volume (in cells' widths) that one cell's
+    // surrounding cells span, i.e. the candidates of an atom in units of natoms
+    auto grid = [&](int div, int* ncell, int* K) {
+      double span = 1.0;
+      for (int d = 0; d < 3; ++d) {
+        int n = (int)std::floor(div * width[d] / cellmin);
+        if (n < 1) n = 1;
+        if (n > 256) n = 256;
+        ncell[d] = n;
+        K[d] = (int)std::ceil(cellmin * n / width[d]);
+        if (K[d] < 1) K[d] = 1;
+        span *= (2.0 * K[d] + 1.0) / n;
+      }
+      return span;
+    };
+    const double span = grid(1, g.ncell, g.K);
+    for (int d = 0; d < 3; ++d)
       if (g.K[d] > 64) {
         set_error("cell narrower than r_c/64: too many periodic images");
         return DP_E_ARG;
       }
-      total *= n;
+    if (fine) {
+      // Half-width cells where whole ones fit the box badly: a box of 1.9 r_c has one cell a side and its
+      // atoms test 27 boxes full of candidates, 5.8 times as many as with r_c / 2 cells.  Where both
+      // grids fit alike (a factor of 1.7) the wider cells serve more centre atoms per staged stream.
+      int n2[3], K2[3];
+      const double span2 = grid(2, n2, K2);
+      const long noff2 = (2L * K2[0] + 1) * (2 * K2[1] + 1) * (2 * K2[2] + 1);
+      if (span >= 1.8 * span2 && noff2 * cfg.ntypes <= kMaxRanges)
+        for (int d = 0; d < 3; ++d) {
+          g.ncell[d] = n2[d];
+          g.K[d] = K2[d];
+        }
     }
-    (void)total;
     // candidate buffer: twice the mean neighbour count of this density, plus a margin
     const double expect = natoms / vol * (4.0 / 3.0) * 3.141592653589793 * rc * rc * rc;
     g.cap = (int)(2.0 * expect + 32.0);
@@ -1244,16 +1297,22 @@ cudaError_t launch_nlist_build(const NlLaunch& L, int ntypes, const double* coor
   const float4* sorted_l = sc.sorted_l;
   const int4* sorted_m = sc.sorted_m;
   const int nkeys = L.ncells_total * ntypes;
-  cudaError_t e = cudaMemsetAsync(cell_count, 0, sizeof(int) * nkeys, st);
+  cudaError_t e = cudaSuccess;
+  if (!(ex && ex->counts_clear)) e = cudaMemsetAsync(cell_count, 0, sizeof(int) * nkeys, st);
   if (e != cudaSuccess) return e;
   const int nb = (L.natoms + 255) / 256;
+  // binning is FP64 arithmetic, about two operations a clock and SM: small blocks spread it (192 atoms in
+  // one block: 7.8 us)
+  const int bin_threads = 64;
   TypeStartCheck nochk;
   std::memset(&nochk, 0, sizeof(nochk));
-  k_bin<<<nb, 256, 0, st>>>(L.geoms, L.atom_frame, L.cell_off, L.natoms, L.ncells_total, ntypes, coord, type,
+  k_bin<<<(L.natoms + bin_threads - 1) / bin_threads, bin_threads, 0, st>>>(L.geoms, L.atom_frame, L.cell_off, L.natoms, L.ncells_total, ntypes, coord, type,
                             cell_count, sc.atom_key, sc.atom_l, sc.atom_m, status, ex ? ex->boxes : nullptr,
                             ex ? ex->nframes : 0, ex ? ex->tshift : nullptr);
   if (nkeys <= 8192) {  // few keys: each fill block scans the counts itself (one launch fewer; nlist_launches)
-    k_fill_scan<<<nb, 256, (size_t)(nkeys + 1) * sizeof(int), st>>>(
+    // wider blocks for many keys: each thread scans up to eight of them
+    const int ft = nkeys <= 2048 ? 256 : 1024;
+    k_fill_scan<<<(L.natoms + ft - 1) / ft, ft, (size_t)(nkeys + 1) * sizeof(int), st>>>(
         L.natoms, cell_count, nkeys, cell_start, sc.atom_key, sc.atom_l, sc.atom_m, sc.sorted_l, sc.sorted_m,
         ex ? ex->perm : nullptr, ex ? ex->type_start : nullptr, L.ncells_total, ntypes, status, ex ? ex->chk : nochk);
   } else {
@@ -1263,27 +1322,42 @@ cudaError_t launch_nlist_build(const NlLaunch& L, int ntypes, const double* coor
                                ntypes, status, ex ? ex->chk : nochk);
   }
   const int cap = L.cap <= 128 ? 128 : (L.cap <= 256 ? 256 : (L.cap <= 512 ? 512 : 1024));
+  const int ccap = std::min(L.cap <= 128 ? 128 : std::max(256, (L.cap + 63) & ~63), 1024);  // the cell kernel's
   // cell-centred search, one CTA per cell, when a cell's candidate stream fits shared memory:
   // room for 1.25 times the mean stream of a cell plus each type's padding (a cell with more
   // reports a capacity error, and the call is retried on the per-atom kernel below)
   const double mean_stream = L.max_stream > 0 ? (double)L.max_stream
                                               : (double)L.natoms / std::max(1, L.ncells_total) * std::max(1, L.max_noff);
   const int S = std::max(1024, ((int)(1.25 * mean_stream) + 64 * ntypes + 64 + 127) & ~127);
-  const size_t csm = cell_smem_bytes(cap, S);
-  if (L.max_noff > 0 && (long)L.max_noff * ntypes <= kMaxRanges && cap <= 512 && csm <= 160 * 1024 && S < 65536) {
+  const size_t csm = cell_smem_bytes(ccap, S);
+  if (L.max_noff > 0 && (long)L.max_noff * ntypes <= kMaxRanges && ccap <= 512 && csm <= 160 * 1024 && S < 65536) {
+    // Centre atoms per block: one a warp (8) or two (16) when the grid then still fits the chip at once
+    // (192 atoms: 37 -> 17 us), else a whole cell, up to three a warp (a cell of a box barely wider than r_c
+    // holds hundreds of atoms, and one block for all of them left the rest of the chip waiting).
+    const double mean = L.max_cell_atoms > 0 ? L.max_cell_atoms : (double)L.natoms / std::max(1, L.ncells_total);
+    const long slots = (long)sm_count() * std::max<long>(1, std::min<long>(4, (long)(227 * 1024 / (csm + 6 * 1024))));
+    int per_block = mean <= 32.0 ? 48 : 24;
+    for (int q = 16; q >= 8; q -= 8)
+      if (L.ncells_total * (long)std::ceil(mean / q) <= slots) per_block = q;
+    const int parts = std::max(1, std::min(64, (int)std::ceil(1.25 * mean / per_block)));
 #define DPGB_NLC_LAUNCH(C)                                                                                       \
   do {                                                                                                           \
     e = allow_max_smem(k_nlist_cell<C>);                                                                         \
     if (e != cudaSuccess) return e;                                                                              \
-    k_nlist_cell<C><<<L.ncells_total, kCellWarps * 32, csm, st>>>(L.geoms, L.cell_off, L.nframes,               \
-                                                                  L.ncells_total, ntypes, coord, cell_start,     \
-                                                                  sorted_l, sorted_m, S, nl_j, nl_code, counts,  \
-                                                                  ex ? ex->disp : nullptr, status);              \
+    k_nlist_cell<C><<<dim3(L.ncells_total, parts), kCellWarps * 32, csm, st>>>(                                  \
+        L.geoms, L.cell_off, L.nframes, L.ncells_total, ntypes, coord, cell_start, sorted_l, sorted_m, S, nl_j,    \
+        nl_code, counts, ex ? ex->disp : nullptr, per_block, ex && ex->lean, status);                            \
   } while (0)
-    if (cap == 128)
+    if (ccap <= 128)
       DPGB_NLC_LAUNCH(128);
-    else if (cap == 256)
+    else if (ccap <= 256)
       DPGB_NLC_LAUNCH(256);
+    else if (ccap <= 320)
+      DPGB_NLC_LAUNCH(320);
+    else if (ccap <= 384)
+      DPGB_NLC_LAUNCH(384);
+    else if (ccap <= 448)
+      DPGB_NLC_LAUNCH(448);
     else
       DPGB_NLC_LAUNCH(512);
 #undef DPGB_NLC_LAUNCH
