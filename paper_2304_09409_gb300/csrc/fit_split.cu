@@ -5,17 +5,32 @@
 //
 // Per tile the CTA runs the chain of GEMMs of the net: forward layers z_l = y_{l-1} W_l + b_l,
 // t_l = tanh z_l, y_l = t_l (+ y_{l-1}), E = y_last . w + b; backward gz_last = w (1 - t_last^2),
-// gy_{l-1} = gz_l W_l^T (+ gy_l), gz_{l-1} = gy_{l-1} (1 - t_{l-1}^2), dE/dD = gz_0 W_0^T.  Each GEMM
-// streams its A operand (the descriptor, or the previous phase's activations) and its weights
-// through one two-stage TMA ring of high and low halves (96 KB a stage); the accumulator lives in
-// tensor memory.  Activations go from each epilogue to the next phase through a per-tile scratch
-// that stays in L2 (high and low BF16 halves for the next A operand, FP32 for the gates): the
-// epilogue writes the next A operand into the idle ring in the swizzled layout of the TMA box and
-// stores it with four tiled TMA stores per half (coalesced), clipped at the end of the tile's
-// type; the FP32 residual stream stays in tensor memory; dE/dD leaves in 256-column chunks from two
-// alternating accumulators, so that one chunk's epilogue overlaps the next chunk's MMAs.  One
-// thread issues TMA, one issues tcgen05.mma, sixteen warps run the epilogues; every mbarrier wait
-// is bounded (on time-out the CTA records an error and finishes).
+// gy_{l-1} = gz_l W_l^T (+ gy_l), gz_{l-1} = gy_{l-1} (1 - t_{l-1}^2), dE/dD = gz_0 W_0^T.
+//
+// What bounds it is the chain: one tile per SM, every phase's MMAs (2.9 us at K = 240) and the epilogue
+// between two phases (7-9 us) follow each other.  So nothing else may stand in that chain:
+//   - the activations stay in shared memory: an epilogue writes the next phase's A operand, high and low
+//     BF16 halves in the tensor core's 128-byte-swizzled layout, 64 columns at a time, and the next
+//     phase's MMAs start on each 64-column block as soon as it is written (two accumulators in tensor
+//     memory, phases alternate);
+//   - weights come through a ring of their own, 32 columns of K a slot (64-byte swizzle; 64 columns of
+//     high and low halves for 240 outputs would not fit twice beside the operand), filled during the
+//     epilogue before;
+//   - the descriptor of the first phase streams through four stages over the whole buffer, which the
+//     operand and the ring then take over;
+//   - the FP32 residual stream (y_l, gy_l) and the gates 1 - t^2 go to an L2-resident scratch that the
+//     thread that wrote them reads back.
+// dE/dD leaves in 192-column chunks from two accumulators, so that a chunk's epilogue overlaps the next
+// one's MMAs.  To have two of 192 columns in tensor memory and five weight slots in shared memory, the
+// chunks' operand gz_0 is split: its high half goes to tensor memory (the MMA reads A from there), its low
+// half to shared memory.  With M_< = 16 each 16-column piece is one m of dE/dD[m][l] and is folded into
+// dE/dT at once, T_< of a thread's row in registers.
+// One tile on 12,288 water atoms, thousand clocks (first GEMM; five epilogues; the four GEMMs between them;
+// chunks; end): 56; 85; 43; 86; 11 (147 us) when each epilogue stored its operand to L2 for the next phase
+// to load, now 47; 64; 22; 66; 3 (107 us).  The first GEMM is at the shared memory's bandwidth, the
+// epilogues at about half their instruction issue.
+// One thread issues TMA, one issues tcgen05.mma, eight warps run the epilogues; every mbarrier wait is
+// bounded (on time-out the CTA records an error and finishes).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -37,22 +52,44 @@ constexpr int kSThreads = kSEpi + 64;    // + a TMA producer warp and an MMA war
 constexpr int kProd = kSEpi / 32, kMmaW = kProd + 1;  // their warp indices
 constexpr int kParts = kSEpi / 128;      // epilogue warps sharing a row quarter, interleaved by 16 columns
 constexpr int kStep = 16 * kParts;       // column stride of one epilogue thread
-constexpr int SBM = 128, SBK = 64;
-constexpr int kSRing = 2;
-constexpr uint32_t kSA = SBM * SBK * 2;   // 16 KB: one 128 x 64 BF16 block of A
-constexpr uint32_t kSB = 256 * SBK * 2;   // 32 KB: up to 256 weight rows
-constexpr uint32_t kSStage = 2 * (kSA + kSB);  // [A hi | A lo | B hi | B lo]
-constexpr int kSLd = 256;  // row pitch of the activation scratch (elements)
+constexpr int SBM = 128;
+constexpr int kKB = 32;                   // K columns of one weight slot (64 bytes a row)
+constexpr uint32_t kOpBlock = SBM * 128;  // 16 KB: 64 columns of one half of the operand
+constexpr uint32_t kOpBytes = 8 * kOpBlock;  // operand: four blocks of the high half, four of the low half
+constexpr uint32_t kDHalf = SBM * kKB * 2;   // 8 KB: 32 descriptor columns of one half
+constexpr int kP0 = 4;                    // stages of the first phase
+constexpr int CH = 192;                   // dE/dD chunk width
+constexpr uint32_t kCHalf = CH * kKB * 2; // 12 KB: 32 columns of K of a chunk's weights, one half
+constexpr int kCRing = 5;                 // chunk weight slots (high and low half each)
+// two slots over the high half of the chain's operand, three behind the low half
+__host__ __device__ constexpr uint32_t chunk_slot(int s) {
+  return (s < 2 ? 0u : kOpBytes - 2u * 2u * kCHalf) + (uint32_t)s * 2u * kCHalf;
+}
+constexpr int kSLd = 256;  // row pitch of the residual and gate scratch (elements)
+
+// Weight rows of a chain slot (the widest layer) and ring slots; chunk slots that fit.
+__host__ __device__ constexpr int slot_rows(int maxw) { return maxw <= 240 ? 240 : 256; }
+__host__ __device__ constexpr int ring_slots(int rows) { return rows == 240 ? 3 : 2; }
+__host__ __device__ constexpr int chunk_slots(int rows) { return rows == 240 ? kCRing : kCRing - 1; }
+__host__ __device__ constexpr uint32_t slot_bytes(int rows) { return 2u * (uint32_t)rows * kKB * 2u; }
+__host__ __device__ constexpr uint32_t buffer_bytes(int rows) {
+  return kOpBytes + (uint32_t)ring_slots(rows) * slot_bytes(rows);
+}
+static_assert(chunk_slot(1) + 2 * kCHalf <= kOpBytes / 2, "two chunk slots fit the operand's high half");
+static_assert(chunk_slot(chunk_slots(240)) <= buffer_bytes(240) && chunk_slot(chunk_slots(256)) <= buffer_bytes(256),
+              "chunk slots fit");
+static_assert(kP0 * (2 * kDHalf + slot_bytes(240)) <= buffer_bytes(240), "first-phase stages fit the buffer");
+static_assert(kP0 * (2 * kDHalf + slot_bytes(256)) <= buffer_bytes(256), "first-phase stages fit the buffer");
 
 struct SplitMaps {
-  CUtensorMap d[2];                       // D hi / lo [rows][KD], box {64, 128}
-  CUtensorMap x[2][2];                    // activation scratch buffer b (hi / lo) [rows][kSLd], box {64, 128}
-  CUtensorMap xt[DP_MAX_TYPES][2][2];     // the same per type, over the type's rows only (stores)
-  CUtensorMap w[DP_MAX_TYPES][2 * kSL][2];  // per type: forward W_l^T (slot l), backward W_l (slot nh + l); hi / lo
+  CUtensorMap d[2];                         // D hi / lo [rows][KD], box {32, 128}
+  // per type, hi / lo: forward W_l^T (slot l), backward W_l (slot nh + l, l >= 1), box {32, outputs}; W_0 for
+  // the chunks (slot nh), box {32, 192}
+  CUtensorMap w[DP_MAX_TYPES][2 * kSL][2];
 };
 
 struct SplitArgs {
-  int ntypes, nh;
+  int ntypes, nh, rows;  // rows of a weight slot
   int width[kSL + 1];  // width[0] = KD, width[l + 1] = outputs of hidden layer l
   int skip[kSL];
   int row_start[DP_MAX_TYPES + 1];
@@ -60,8 +97,11 @@ struct SplitArgs {
   const float* bias[DP_MAX_TYPES][kSL];
   const float* w_last[DP_MAX_TYPES];
   float b_last[DP_MAX_TYPES];
-  __nv_bfloat16* xs[2][2];  // activation scratch [2 buffers][hi, lo] [rows][kSLd]
-  float* gate;              // 1 - t_l^2 of the inner hidden layers [nh][rows][kSLd]
+  // scratch of every tile, each value read back by the thread that wrote it: 8-column groups, a row's
+  // eight values in one 32-byte sector and the rows of a group contiguous (a warp's access covers 8 lines;
+  // with a row pitch of 256 columns it covered 32, and the L1 tag rate bound the epilogues)
+  float* resid;             // y_l forward, gy_l backward [tiles][32][128][8]
+  float* gate;              // 1 - t_l^2 of the inner hidden layers [nh][tiles][32][128][8]
   const int* perm;
   double* atom_e;
   float* gD;                // dE/dD FP32 [rows][KD], or null when gT is formed instead
@@ -111,11 +151,20 @@ __global__ void __launch_bounds__(kSThreads, 1) k_fit_split(const __grid_constan
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kSRing * kSStage);
-  uint64_t* empty = full + kSRing;
-  uint64_t* accf = empty + kSRing;  // [2] accumulator buffer ready (MMA -> epilogue)
-  uint64_t* accfree = accf + 2;     // [2] accumulator read and phase outputs written (epilogue -> MMA, TMA)
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(accfree + 2);
+  const uint32_t slotb = slot_bytes(g.rows), halfb = slotb / 2;
+  const int NS = ring_slots(g.rows);
+  unsigned char* ring = smem + kOpBytes;
+  uint64_t* full0 = reinterpret_cast<uint64_t*>(smem + buffer_bytes(g.rows));
+  uint64_t* empty0 = full0 + kP0;
+  uint64_t* fullw = empty0 + kP0;   // [3]
+  uint64_t* emptyw = fullw + 3;     // [3]
+  uint64_t* accf = emptyw + 3;      // [2] accumulator ready (MMA -> epilogue)
+  uint64_t* accfree = accf + 2;     // [2] dE/dD chunk read (epilogue -> MMA)
+  uint64_t* aready = accfree + 2;   // [4] 64-column block of the next operand written (epilogue -> MMA)
+  uint64_t* chain_done = aready + 4;  // every MMA of the chain phases has completed
+  uint64_t* fullc = chain_done + 1;   // [kCRing]
+  uint64_t* emptyc = fullc + kCRing;  // [kCRing]
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(emptyc + kCRing + 1);
   float* s_e = reinterpret_cast<float*>(tmem_holder + 4);  // [kParts][128]
   float* s_bias = s_e + kParts * SBM;                      // [kSL][256] biases of the hidden layers
   float* s_wl = s_bias + kSL * 256;                        // [256] weights of the output layer
@@ -127,18 +176,30 @@ __global__ void __launch_bounds__(kSThreads, 1) k_fit_split(const __grid_constan
   const int row_end = g.row_start[t + 1];
   const long rows = g.row_start[g.ntypes];
   const int nh = g.nh, KD = g.width[0];
-  const int nch = (KD + 255) / 256;
-  // phases: forward layers 0 .. nh-1, backward layers nh-1 .. 1, then the nch dE/dD chunks
-  const int nphase = nh + (nh - 1) + nch;
+  const int nch = (KD + CH - 1) / CH;
+  // chain phases: forward layers 0 .. nh-1, backward layers nh-1 .. 1; phase p accumulates in tensor-memory
+  // columns [256 (p & 1), ..).  The last one is even; its epilogue puts the high half of the chunks' operand
+  // into columns [384, 512), and chunk c accumulates in columns [192 (c & 1), ..).
+  const int nchain = 2 * nh - 1;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kSRing; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+    for (int s = 0; s < kP0; ++s) {
+      mbar_init(&full0[s], 1);
+      mbar_init(&empty0[s], 1);
+    }
+    for (int s = 0; s < 3; ++s) {
+      mbar_init(&fullw[s], 1);
+      mbar_init(&emptyw[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accf[b], 1);
       mbar_init(&accfree[b], kSEpi);
+    }
+    for (int b = 0; b < 4; ++b) mbar_init(&aready[b], kSEpi);
+    mbar_init(chain_done, 1);
+    for (int s = 0; s < kCRing; ++s) {
+      mbar_init(&fullc[s], 1);
+      mbar_init(&emptyc[s], 1);
     }
     mbar_fence_init();
   }
@@ -148,135 +209,186 @@ __global__ void __launch_bounds__(kSThreads, 1) k_fit_split(const __grid_constan
   tc_fence_after();
   const uint32_t tmem = *tmem_holder;
 
-  // phase p: its GEMM (K, N), the A map pair, the weight slot, the accumulator buffer, and
-  // whether its A operand was written by the phase before (the producer then waits for it)
-  auto phase_info = [&](int p, int& K, int& N, const CUtensorMap*& ah, const CUtensorMap*& al, int& wslot, int& wrow,
-                        int& buf) {
-    buf = 0;
-    wrow = 0;
-    if (p < nh) {  // forward layer p: A = D (p == 0) or the scratch the previous layer wrote
+  // chain phase p >= 1: its GEMM (K, N) and weight map
+  auto phase_info = [&](int p, int& K, int& N, int& wslot) {
+    if (p < nh) {
       K = g.width[p];
       N = g.width[p + 1];
-      ah = p == 0 ? &mp.d[0] : &mp.x[(p - 1) & 1][0];
-      al = p == 0 ? &mp.d[1] : &mp.x[(p - 1) & 1][1];
       wslot = p;
-    } else if (p < 2 * nh - 1) {  // backward layer l = nh - 1 - (p - nh): A = gz_l
+    } else {  // backward layer l = nh - 1 - (p - nh): A = gz_l
       const int l = nh - 1 - (p - nh);
       K = g.width[l + 1];
       N = g.width[l];
-      const int xb = (p - 1) & 1;
-      ah = &mp.x[xb][0];
-      al = &mp.x[xb][1];
       wslot = nh + l;
-    } else {  // dE/dD chunk c = gz_0 W_0^T, columns [256 c, 256 c + 256)
-      const int c = p - (2 * nh - 1);
-      K = g.width[1];
-      N = min(256, KD - 256 * c);
-      const int xb = (2 * nh - 2) & 1;
-      ah = &mp.x[xb][0];
-      al = &mp.x[xb][1];
-      wslot = nh;
-      wrow = 256 * c;
-      buf = c & 1;
     }
   };
+  const int nkc = (g.width[1] + kKB - 1) / kKB;  // weight slots' worth of a chunk
+  const int NC = chunk_slots(g.rows);
+  const uint32_t p0_stage = 2 * kDHalf + slotb;
+  const int nk0 = (KD + kKB - 1) / kKB;
 
   if (warp == kProd) {
     if (lane == 0) {
       // ---- TMA producer ----
-      int it = 0;
       bool ok = true;
-      int fr[2] = {0, 0};  // accumulator-free phases waited for, per buffer
-      for (int p = 0; ok && p < nphase; ++p) {
-        int K, N, wslot, wrow, buf;
-        const CUtensorMap *ah, *al;
-        phase_info(p, K, N, ah, al, wslot, wrow, buf);
-        // the A operand of phases after the first was written by the previous phase's epilogue
-        if (p >= 1 && p <= 2 * nh - 1) {
-          const int pb = 0;  // chain phases use accumulator buffer 0
-          ok = mbar_wait(&accfree[pb], fr[pb] & 1, g.err);
-          ++fr[pb];
-          if (!ok) break;
+      int n0 = 0, it = 0;  // loads issued: first phase, weight ring
+      for (int kb = 0; kb < nk0; ++kb) {
+        const int s = kb % kP0;
+        if (kb >= kP0 && !mbar_wait(&empty0[s], ((kb / kP0) - 1) & 1, g.err)) {
+          ok = false;
+          break;
         }
-        const int nkb = (K + SBK - 1) / SBK;
-        for (int kb = 0; ok && kb < nkb; ++kb) {
-          const int s = it % kSRing;
-          if (it >= kSRing && !mbar_wait(&empty[s], ((it / kSRing) - 1) & 1, g.err)) {
+        unsigned char* st = smem + s * p0_stage;
+        mbar_expect_tx(&full0[s], 2 * kDHalf + 2u * (uint32_t)g.width[1] * kKB * 2u);
+        tma_load_2d(st, &mp.d[0], &full0[s], kb * kKB, row0);
+        tma_load_2d(st + kDHalf, &mp.d[1], &full0[s], kb * kKB, row0);
+        tma_load_2d(st + 2 * kDHalf, &mp.w[t][0][0], &full0[s], kb * kKB, 0);
+        tma_load_2d(st + 2 * kDHalf + halfb, &mp.w[t][0][1], &full0[s], kb * kKB, 0);
+        n0 = kb + 1;
+      }
+      // the ring lies over the first phase's stages: they are free once its MMAs have completed
+      if (ok) ok = mbar_wait(&accf[0], 0, g.err);
+      for (int p = 1; ok && p < nchain; ++p) {
+        int K, N, wslot;
+        phase_info(p, K, N, wslot);
+        const int nkb = (K + kKB - 1) / kKB;
+        for (int kb = 0; kb < nkb; ++kb, ++it) {
+          const int s = it % NS;
+          if (it >= NS && !mbar_wait(&emptyw[s], ((it / NS) - 1) & 1, g.err)) {
             ok = false;
             break;
           }
-          unsigned char* st = smem + s * kSStage;
-          // the weight boxes hold N rows (chain layers) or 256 (dE/dD chunks; rows beyond W_0 are zero-filled)
-          const uint32_t brows = p < 2 * nh - 1 ? (uint32_t)N : 256u;
-          mbar_expect_tx(&full[s], 2 * kSA + 2 * brows * 128u);
-          tma_load_2d(st, ah, &full[s], kb * SBK, row0);
-          tma_load_2d(st + kSA, al, &full[s], kb * SBK, row0);
-          tma_load_2d(st + 2 * kSA, &mp.w[t][wslot][0], &full[s], kb * SBK, wrow);
-          tma_load_2d(st + 2 * kSA + kSB, &mp.w[t][wslot][1], &full[s], kb * SBK, wrow);
-          ++it;
+          unsigned char* st = ring + s * slotb;
+          mbar_expect_tx(&fullw[s], 2u * (uint32_t)N * kKB * 2u);
+          tma_load_2d(st, &mp.w[t][wslot][0], &fullw[s], kb * kKB, 0);
+          tma_load_2d(st + halfb, &mp.w[t][wslot][1], &fullw[s], kb * kKB, 0);
         }
       }
+      // the chunks' slots lie over everything the chain used
+      if (ok) ok = mbar_wait(chain_done, 0, g.err);
+      int nc_ = 0;
+      for (int c = 0; ok && c < nch; ++c)
+        for (int kb = 0; kb < nkc; ++kb) {
+          const int s = nc_ % NC;
+          if (nc_ >= NC && !mbar_wait(&emptyc[s], ((nc_ / NC) - 1) & 1, g.err)) {
+            ok = false;
+            break;
+          }
+          unsigned char* st = smem + chunk_slot(s);
+          mbar_expect_tx(&fullc[s], 2 * kCHalf);  // rows beyond W_0 are zero-filled
+          tma_load_2d(st, &mp.w[t][nh][0], &fullc[s], kb * kKB, CH * c);
+          tma_load_2d(st + kCHalf, &mp.w[t][nh][1], &fullc[s], kb * kKB, CH * c);
+          ++nc_;
+        }
       // every copy this thread started has landed before the CTA may exit
-      for (int s = 0; s < kSRing && s < it; ++s) {
-        const int last = s + kSRing * ((it - 1 - s) / kSRing);
-        mbar_wait(&full[s], (last / kSRing) & 1, g.err);
-      }
+      for (int kb = max(0, n0 - kP0); kb < n0; ++kb) mbar_wait(&full0[kb % kP0], (kb / kP0) & 1, g.err);
+      for (int k = max(0, it - NS); k < it; ++k) mbar_wait(&fullw[k % NS], (k / NS) & 1, g.err);
+      for (int k = max(0, nc_ - NC); k < nc_; ++k) mbar_wait(&fullc[k % NC], (k / NC) & 1, g.err);
     }
   } else if (warp == kMmaW) {
-    if (lane == 0) {
-      // ---- MMA issuer ----
-      int it = 0;
+    {
+      // ---- MMA issuer: the whole warp runs the loop, one lane issues ----
+      const uint32_t by = elect_lane();
       bool ok = true;
-      int fr[2] = {0, 0};
-      for (int p = 0; ok && p < nphase; ++p) {
-        int K, N, wslot, wrow, buf;
-        const CUtensorMap *ah, *al;
-        phase_info(p, K, N, ah, al, wslot, wrow, buf);
-        // the accumulator buffer must have been read by the epilogue of its previous phase
-        if (p >= 1) {
-          int need;
-          if (p <= 2 * nh - 1) {
-            need = 1;  // chain: the previous phase's epilogue
-          } else {
-            const int c = p - (2 * nh - 1);
-            need = (buf == 0) ? 1 : (c >= 2 ? 1 : 0);  // buffer 0 follows the chain; buffer 1 from chunk 3 on
-          }
-          if (need) {
-            ok = mbar_wait(&accfree[buf], fr[buf] & 1, g.err);
-            ++fr[buf];
-            if (!ok) break;
-          }
-        }
-        tc_fence_after();
-        const uint32_t idesc = idesc_f16(SBM, N <= 256 ? ((N + 15) & ~15) : 256, 1);
-        const uint32_t acc = tmem + (uint32_t)(buf * 256);
-        const int nkb = (K + SBK - 1) / SBK;
-        for (int kb = 0; kb < nkb; ++kb) {
-          const int s = it % kSRing;
-          if (!mbar_wait(&full[s], (it / kSRing) & 1, g.err)) {
+      // three passes of one 16-column step: small terms first (lo.hi, hi.lo, then hi.hi)
+      auto step = [&](uint32_t acc, uint64_t ah, uint64_t al, uint64_t bh, uint64_t bl, uint32_t idesc, bool first) {
+        mma_f16_by(by, acc, al, bh, idesc, first ? 0 : 1);
+        mma_f16_by(by, acc, ah, bl, idesc, 1);
+        mma_f16_by(by, acc, ah, bh, idesc, 1);
+      };
+      {
+        const uint32_t idesc = idesc_f16(SBM, g.width[1], 1);
+        for (int kb = 0; kb < nk0; ++kb) {
+          const int s = kb % kP0;
+          if (!mbar_wait(&full0[s], (kb / kP0) & 1, g.err)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t sa = su32(smem + s * kSStage);
-          const uint64_t ah_ = sdesc_sw128(sa), al_ = sdesc_sw128(sa + kSA);
-          const uint64_t bh_ = sdesc_sw128(sa + 2 * kSA), bl_ = sdesc_sw128(sa + 2 * kSA + kSB);
+          const uint32_t sa = su32(smem + s * p0_stage);
+          const uint64_t ah = sdesc_sw64(sa), al = sdesc_sw64(sa + kDHalf);
+          const uint64_t bh = sdesc_sw64(sa + 2 * kDHalf), bl = sdesc_sw64(sa + 2 * kDHalf + halfb);
 #pragma unroll
-          for (int k = 0; k < SBK / 16; ++k) {  // small terms first: lo.hi, hi.lo, then hi.hi
-            mma_f16(acc, al_ + 2 * k, bh_ + 2 * k, idesc, (kb | k) != 0);
-            mma_f16(acc, ah_ + 2 * k, bl_ + 2 * k, idesc, 1);
-            mma_f16(acc, ah_ + 2 * k, bh_ + 2 * k, idesc, 1);
-          }
-          mma_commit(&empty[s]);
-          ++it;
+          for (int k = 0; k < kKB / 16; ++k)
+            step(tmem, ah + 2 * k, al + 2 * k, bh + 2 * k, bl + 2 * k, idesc, (kb | k) == 0);
+          mma_commit_by(by, &empty0[s]);
         }
-        mma_commit(&accf[buf]);
+        mma_commit_by(by, &accf[0]);
+      }
+      int it = 0;
+      uint32_t free_par = 0, ready_par = 0;  // parities of the waits below, one bit per barrier
+      if (nchain == 1) mma_commit_by(by, chain_done);
+      for (int p = 1; ok && p < nchain; ++p) {
+        int K, N, wslot;
+        phase_info(p, K, N, wslot);
+        const int buf = p & 1;
+        // (the accumulator was last read two phases ago, by an epilogue that the operand blocks below have
+        // waited for)
+        const uint32_t idesc = idesc_f16(SBM, N, 1);
+        const uint32_t acc = tmem + (uint32_t)(buf * 256);
+        const int nkb = (K + kKB - 1) / kKB;
+        for (int kb = 0; kb < nkb; ++kb, ++it) {
+          const int s = it % NS;
+          if ((kb & 1) == 0) {
+            if (!mbar_wait(&aready[kb >> 1], (ready_par >> (kb >> 1)) & 1u, g.err)) {
+              ok = false;
+              break;
+            }
+            ready_par ^= 1u << (kb >> 1);
+          }
+          if (!mbar_wait(&fullw[s], (it / NS) & 1, g.err)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t sa = su32(smem + (kb >> 1) * kOpBlock), sw = su32(ring + s * slotb);
+          const uint32_t ko = (uint32_t)(kb & 1) * 4;  // second half of the operand's 64-column block
+          const uint64_t ah = sdesc_sw128(sa) + ko, al = sdesc_sw128(sa + 4 * kOpBlock) + ko;
+          const uint64_t bh = sdesc_sw64(sw), bl = sdesc_sw64(sw + halfb);
+#pragma unroll
+          for (int k = 0; k < kKB / 16; ++k)
+            step(acc, ah + 2 * k, al + 2 * k, bh + 2 * k, bl + 2 * k, idesc, (kb | k) == 0);
+          mma_commit_by(by, &emptyw[s]);
+        }
+        mma_commit_by(by, &accf[buf]);
+        if (p == nchain - 1) mma_commit_by(by, chain_done);
+      }
+      // chunks: the operand is complete (and the last chain accumulator, whose columns they take, is read)
+      for (int kb = 0; ok && 2 * kb < nkc; ++kb) ok = mbar_wait(&aready[kb], (ready_par >> kb) & 1u, g.err);
+      tc_fence_after();
+      int nc_ = 0;
+      for (int c = 0; ok && c < nch; ++c) {
+        const int buf = c & 1;
+        if (c >= 2) {
+          if (!mbar_wait(&accfree[buf], (free_par >> buf) & 1u, g.err)) break;
+          free_par ^= 1u << buf;
+          tc_fence_after();
+        }
+        const uint32_t idesc = idesc_f16(SBM, min(CH, KD - CH * c), 1);
+        const uint32_t acc = tmem + (uint32_t)(buf * CH);
+        for (int kb = 0; kb < nkc; ++kb, ++nc_) {
+          const int s = nc_ % NC;
+          if (!mbar_wait(&fullc[s], (nc_ / NC) & 1, g.err)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t sw = su32(smem + chunk_slot(s)), ah = tmem + 384u + (uint32_t)kb * 16u;
+          const uint64_t al = sdesc_sw128(su32(smem + (4 + (kb >> 1)) * kOpBlock)) + (uint32_t)(kb & 1) * 4;
+          const uint64_t bh = sdesc_sw64(sw), bl = sdesc_sw64(sw + kCHalf);
+#pragma unroll
+          for (int k = 0; k < kKB / 16; ++k) {
+            mma_f16_by(by, acc, al + 2 * k, bh + 2 * k, idesc, (kb | k) != 0);
+            mma_f16_ta_by(by, acc, ah + 8 * k, bl + 2 * k, idesc, 1);
+            mma_f16_ta_by(by, acc, ah + 8 * k, bh + 2 * k, idesc, 1);
+          }
+          mma_commit_by(by, &emptyc[s]);
+        }
+        mma_commit_by(by, &accf[buf]);
       }
     }
   } else {
   // ---- epilogues: warps w and w + 4 own rows 32(w % 4) .. +31 and take 16-column pieces in turn ----
-  // The FP32 residual stream (y_l forward, gy_l backward) stays in tensor-memory columns
-  // [256, 512) of the thread's row, which the chain phases leave free.
   const int quad = warp & 3, part = warp >> 2;
   const int rl = quad * 32 + lane;
   const long row = row0 + rl;
@@ -290,44 +402,46 @@ __global__ void __launch_bounds__(kSThreads, 1) k_fit_split(const __grid_constan
     __syncwarp();
     tc_fence_after();
   };
-  auto release = [&](int buf, bool stored) {
-    if (stored) tmem_wait_st();
-    fence_async_global();  // this phase's global writes, read next by TMA
-    tc_fence_before();
-    mbar_arrive(&accfree[buf]);
+  constexpr int kGroup = SBM * 8;  // floats of an 8-column group
+  float* res = g.resid + (long)blockIdx.x * (SBM * kSLd) + rl * 8;
+  auto gate_of = [&](int l) -> float* {
+    return g.gate + ((long)l * gridDim.x + blockIdx.x) * (SBM * kSLd) + rl * 8;
   };
-  auto gate_at = [&](int l, int col) -> float* { return g.gate + ((long)l * rows + row) * kSLd + col; };
-  // the next A operand, staged in the idle ring: 64-column block kb of half hl at (2 kb + hl) * kSA,
-  // row rl at rl * 128 bytes, 16-byte chunk j at (j ^ (rl % 8)) * 16 (the TMA box's 128-byte swizzle)
-  auto put_x = [&](int c, const float* x) {
+  // the next A operand: 64-column block kb of the high half at kb * kOpBlock, of the low half four blocks
+  // further, row rl at rl * 128 bytes, 16-byte chunk j at (j ^ (rl % 8)) * 16 (128-byte swizzle); the chunks'
+  // high half to tensor memory
+  auto put_x = [&](int c, const float* x, bool chunks) {
     __align__(16) __nv_bfloat16 hi[16], lo[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) split2(x[i], hi[i], lo[i]);
     const int kb = c >> 6, j = (c & 63) >> 3;
-    unsigned char* bh = smem + (2 * kb) * kSA + rl * 128;
-    unsigned char* bl = bh + kSA;
-    *reinterpret_cast<uint4*>(bh + ((j ^ (rl & 7)) << 4)) = *reinterpret_cast<const uint4*>(hi);
-    *reinterpret_cast<uint4*>(bh + (((j + 1) ^ (rl & 7)) << 4)) = *reinterpret_cast<const uint4*>(hi + 8);
+    unsigned char* bh = smem + kb * kOpBlock + rl * 128;
+    unsigned char* bl = bh + 4 * kOpBlock;
+    if (chunks) {
+      tmem_st8(tq + 384 + (c >> 1), reinterpret_cast<const uint32_t*>(hi));
+      tmem_wait_st();
+    } else {
+      *reinterpret_cast<uint4*>(bh + ((j ^ (rl & 7)) << 4)) = *reinterpret_cast<const uint4*>(hi);
+      *reinterpret_cast<uint4*>(bh + (((j + 1) ^ (rl & 7)) << 4)) = *reinterpret_cast<const uint4*>(hi + 8);
+    }
     *reinterpret_cast<uint4*>(bl + ((j ^ (rl & 7)) << 4)) = *reinterpret_cast<const uint4*>(lo);
     *reinterpret_cast<uint4*>(bl + (((j + 1) ^ (rl & 7)) << 4)) = *reinterpret_cast<const uint4*>(lo + 8);
   };
-  // the staged operand to scratch buffer xb, one 64-column block at a time: after its second pieces
-  // of block kb (loop iteration k odd) every thread has staged its part of the block, and one
-  // thread starts the block's two TMA stores while the epilogue goes on; all complete before the
-  // phase is released
-  auto store_block = [&](int k, int xb) {
+  // after this thread's second piece of a 64-column block: its part of the block is written and its
+  // accumulator columns are in registers
+  auto block_done = [&](int k) {
     if (!(k & 1)) return;
-    const int kb = k >> 1;
     fence_async_smem();
-    bar_sync(1, kSEpi);
-    if (threadIdx.x == 0) {
-      for (int hl = 0; hl < 2; ++hl)
-        tma_store_2d(&mp.xt[t][xb][hl], smem + (2 * kb + hl) * kSA, kb * 64, row0 - g.row_start[t]);
-      bulk_commit();
-    }
+    tc_fence_before();
+    mbar_arrive(&aready[k >> 1]);
   };
-  auto flush_wait = [&]() {
-    if (threadIdx.x == 0) bulk_wait0();
+  auto load16 = [&](const float* base, int c, float* y) {
+    ld_v8(base + (c >> 3) * kGroup, y);
+    ld_v8(base + ((c >> 3) + 1) * kGroup, y + 8);
+  };
+  auto store16 = [&](float* base, int c, const float* y) {
+    st_v8(base + (c >> 3) * kGroup, y);
+    st_v8(base + ((c >> 3) + 1) * kGroup, y + 8);
   };
   // biases and output weights of this tile's type into shared memory
   for (int l = 0; l < nh; ++l)
@@ -337,27 +451,31 @@ __global__ void __launch_bounds__(kSThreads, 1) k_fit_split(const __grid_constan
   bar_sync(1, kSEpi);
   // forward
   for (int l = 0; l < nh; ++l) {
-    wait_acc(0);
-    const int N = g.width[l + 1];
+    const int N = g.width[l + 1], nc = (N + 63) & ~63;  // zeros to the next whole block: the operand's K padding
     const bool last = (l == nh - 1), sk = g.skip[l] == 1;
     const float* bias = s_bias + l * 256;
-    const int xb = l & 1;
     float e_acc = 0.f;
     // the accumulator (and residual) pieces load one ahead of the piece being processed
-    uint32_t na[16], ny[16];
-    tmem_ld16_async(tq + part * 16, na);
-    if (sk) tmem_ld16_async(tq + 256 + part * 16, ny);
+    uint32_t na[16];
+    float ny[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) ny[i] = 0.f;
+    if (sk) load16(res, part * 16, ny);
+    wait_acc(l & 1);
+    const uint32_t ta = tq + (uint32_t)((l & 1) * 256);
+    tmem_ld16_async(ta + part * 16, na);
     tmem_wait_ld();
-    for (int c = part * 16, k = 0; c < kSLd; c += kStep, ++k) {  // zeros beyond N: the next A operand's K padding
-      uint32_t ra[16], ry[16];
+    for (int c = part * 16, k = 0; c < nc; c += kStep, ++k) {
+      uint32_t ra[16];
+      float ry[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         ra[i] = na[i];
         ry[i] = ny[i];
       }
-      if (c + kStep < kSLd) {
-        tmem_ld16_async(tq + c + kStep, na);
-        if (sk) tmem_ld16_async(tq + 256 + c + kStep, ny);
+      if (c + kStep < nc) {
+        tmem_ld16_async(ta + c + kStep, na);
+        if (sk && c + kStep < N) load16(res, c + kStep, ny);
       }
       float out[16], y[16], gt[16];
       if (c < N) {  // widths are multiples of 16: a piece is all real columns or all padding
@@ -365,7 +483,7 @@ __global__ void __launch_bounds__(kSThreads, 1) k_fit_split(const __grid_constan
         for (int i = 0; i < 16; ++i) {
           const int col = c + i;
           const float th = tanh_ex(__uint_as_float(ra[i]) + bias[col]);
-          y[i] = th + (sk ? __uint_as_float(ry[i]) : 0.f);
+          y[i] = th + (sk ? ry[i] : 0.f);
           gt[i] = 1.f - th * th;
           if (last) {
             const float w = s_wl[col];
@@ -377,16 +495,15 @@ __global__ void __launch_bounds__(kSThreads, 1) k_fit_split(const __grid_constan
         }
       } else {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) out[i] = y[i] = gt[i] = 0.f;
+        for (int i = 0; i < 16; ++i) out[i] = 0.f;
       }
-      tmem_wait_ld();                          // the next piece has landed
-      if (!last) tmem_st16(tq + 256 + c, y);  // the residual stream of the next layer
-      put_x(c, out);
-      if (rv && !last && c < N) {
-        st_v8(gate_at(l, c), gt);
-        st_v8(gate_at(l, c + 8), gt + 8);
+      tmem_wait_ld();  // the next piece has landed
+      put_x(c, out, nh == 1);
+      block_done(k);
+      if (!last && c < N) {
+        store16(res, c, y);  // the residual stream of the next layer
+        store16(gate_of(l), c, gt);
       }
-      store_block(k, xb);
     }
     if (last) {
       s_e[part * SBM + rl] = e_acc;
@@ -398,62 +515,56 @@ __global__ void __launch_bounds__(kSThreads, 1) k_fit_split(const __grid_constan
         g.atom_e[g.perm[row]] = (double)(e + g.b_last[t]);
       }
     }
-    flush_wait();
-    release(0, !last);
   }
-  // backward of layers nh-1 .. 1: gz_{l-1} into the scratch, gy_{l-1} kept for the next skip
+  // backward of layers nh-1 .. 1: gz_{l-1} as the next operand, gy_{l-1} kept for the next skip
   for (int l = nh - 1; l >= 1; --l) {
-    const int N = g.width[l];
-    if (rv)  // this row's gates towards L1 while the GEMM of this phase runs
-      for (int c = part * 16; c < N; c += kStep)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) prefetch_l1(gate_at(l - 1, c + 4 * q));
-    wait_acc(0);
+    const int N = g.width[l], nc = (N + 63) & ~63;
     const bool top = (l == nh - 1), sk = g.skip[l] == 1, keep = (l - 1 >= 1);
     const int p = nh + (nh - 1 - l);  // phase index
-    const int xb = p & 1;
     const bool ldy = sk && !top;
-    uint32_t na[16], ny[16];
-    tmem_ld16_async(tq + part * 16, na);
-    if (ldy) tmem_ld16_async(tq + 256 + part * 16, ny);
+    const float* gates = gate_of(l - 1);
+    uint32_t na[16];
+    float ny[16], ng[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) ny[i] = 0.f;
+    if (ldy) load16(res, part * 16, ny);
+    load16(gates, part * 16, ng);
+    wait_acc(p & 1);
+    const uint32_t ta = tq + (uint32_t)((p & 1) * 256);
+    tmem_ld16_async(ta + part * 16, na);
     tmem_wait_ld();
-    for (int c = part * 16, k = 0; c < kSLd; c += kStep, ++k) {  // zeros beyond N: the next A operand's K padding
-      uint32_t ra[16], ry[16];
+    for (int c = part * 16, k = 0; c < nc; c += kStep, ++k) {
+      uint32_t ra[16];
+      float ry[16], gt[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         ra[i] = na[i];
         ry[i] = ny[i];
+        gt[i] = c < N ? ng[i] : 0.f;
       }
-      if (c + kStep < kSLd) {
-        tmem_ld16_async(tq + c + kStep, na);
-        if (ldy) tmem_ld16_async(tq + 256 + c + kStep, ny);
-      }
-      float gt[16];
-      if (rv && c < N) {
-        ld_v8(gate_at(l - 1, c), gt);
-        ld_v8(gate_at(l - 1, c + 8), gt + 8);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) gt[i] = 0.f;
+      if (c + kStep < nc) {
+        tmem_ld16_async(ta + c + kStep, na);
+        if (c + kStep < N) {
+          if (ldy) load16(res, c + kStep, ny);
+          load16(gates, c + kStep, ng);
+        }
       }
       float gy[16], gz[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         const int col = c + i;
         float v = col < N ? __uint_as_float(ra[i]) : 0.f;
-        if (sk && col < N) v += top ? s_wl[col] : __uint_as_float(ry[i]);
+        if (sk && col < N) v += top ? s_wl[col] : ry[i];
         gy[i] = v;
         gz[i] = v * gt[i];
       }
       tmem_wait_ld();
-      if (keep) tmem_st16(tq + 256 + c, gy);
-      put_x(c, gz);
-      store_block(k, xb);
+      put_x(c, gz, l == 1);
+      block_done(k);
+      if (keep && c < N) store16(res, c, gy);
     }
-    flush_wait();
-    release(0, keep);
   }
-  // dE/dD in 256-column chunks from the two alternating accumulators: stored, or (gT mode, 16-column
+  // dE/dD in chunks of 192 columns from the two alternating accumulators: stored, or (gT mode, 16-column
   // pieces = one m) folded at once into dE/dT, term 1 per piece and term 2 accumulated per row
   const bool gtm = g.gT != nullptr;
   float ext[16][4];
@@ -461,39 +572,30 @@ __global__ void __launch_bounds__(kSThreads, 1) k_fit_split(const __grid_constan
   for (int l = 0; l < 16; ++l)
 #pragma unroll
     for (int q = 0; q < 4; ++q) ext[l][q] = 0.f;
-  // T_< of the tile's rows in shared memory over the forward's dead biases and energies: row rl's
-  // float4 l at rl * 16 + (l ^ (rl % 8)), so that the 32 rows of a warp read without conflicts
-  float4* s_tl = reinterpret_cast<float4*>(s_e);
-  if (gtm) {
-    for (int e = threadIdx.x; e < SBM * 16; e += kSEpi) {
-      const int r = e >> 4, l = e & 15;
-      const long rr = row0 + r;
-      s_tl[r * 16 + (l ^ (r & 7))] = rr < row_end ? __ldg(reinterpret_cast<const float4*>(g.Tm + (rr * g.M + l) * 4))
-                                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    bar_sync(1, kSEpi);
-  }
+  float4 tl[16];  // T_< of this thread's row
+#pragma unroll
+  for (int l = 0; l < 16; ++l)
+    tl[l] = gtm && rv ? __ldg(reinterpret_cast<const float4*>(g.Tm + (row * g.M + l) * 4))
+                      : make_float4(0.f, 0.f, 0.f, 0.f);
   for (int c = 0; c < nch; ++c) {
     const int buf = c & 1;
     wait_acc(buf);
-    const int N = min(256, KD - 256 * c);
-    float* dst = gtm ? nullptr : g.gD + row * KD + 256 * c;
-    const uint32_t tb = tq + (uint32_t)(buf * 256);
+    const int N = min(CH, KD - CH * c);
+    const uint32_t tb = tq + (uint32_t)(buf * CH);
     for (int q = part * 16; q < N; q += kStep) {
       float v[16];
       tmem_ld16(tb + q, v);
       if (rv) {
         if (gtm) {
-          const int m = (256 * c + q) >> 4;
+          const int m = (CH * c + q) >> 4;
           const float4 tm = __ldg(reinterpret_cast<const float4*>(g.Tm + (row * g.M + m) * 4));
           float t1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
           for (int l = 0; l < 16; ++l) {
-            const float4 tl = s_tl[rl * 16 + (l ^ (rl & 7))];
-            t1[0] += v[l] * tl.x;
-            t1[1] += v[l] * tl.y;
-            t1[2] += v[l] * tl.z;
-            t1[3] += v[l] * tl.w;
+            t1[0] += v[l] * tl[l].x;
+            t1[1] += v[l] * tl[l].y;
+            t1[2] += v[l] * tl[l].z;
+            t1[3] += v[l] * tl[l].w;
             ext[l][0] += v[l] * tm.x;
             ext[l][1] += v[l] * tm.y;
             ext[l][2] += v[l] * tm.z;
@@ -501,8 +603,9 @@ __global__ void __launch_bounds__(kSThreads, 1) k_fit_split(const __grid_constan
           }
           reinterpret_cast<float4*>(g.gT)[(long)m * rows + row] = make_float4(t1[0], t1[1], t1[2], t1[3]);
         } else {
-          st_v8(dst + q, v);
-          st_v8(dst + q + 8, v + 8);
+          float* dst = g.gD + row * KD + CH * c + q;
+          st_v8(dst, v);
+          st_v8(dst + 8, v + 8);
         }
       }
     }
@@ -510,26 +613,34 @@ __global__ void __launch_bounds__(kSThreads, 1) k_fit_split(const __grid_constan
     mbar_arrive(&accfree[buf]);
   }
   if (gtm) {
-    // term 2 of the rows' first 16 m: the parts' partial sums meet in the idle ring (every load and
-    // MMA of the tile completed before the last chunk's accumulator became ready)
-    float* s_ext = reinterpret_cast<float*>(smem);  // [kParts][128][64]
+    // term 2 of the rows' first 16 m: the parts' partial sums meet in the operand buffer (every MMA of
+    // the tile completed before the last chunk's accumulator became ready).  A row's dE/dT of m < 16 was
+    // written by the thread of m's parity, which is the one that adds here.
+    float* s_ext = reinterpret_cast<float*>(smem);  // [kParts][128][68]
 #pragma unroll
     for (int l = 0; l < 16; ++l)
-      *reinterpret_cast<float4*>(s_ext + ((part * SBM) + rl) * 64 + l * 4) =
+      *reinterpret_cast<float4*>(s_ext + ((part * SBM) + rl) * 68 + l * 4) =
           make_float4(ext[l][0], ext[l][1], ext[l][2], ext[l][3]);
     bar_sync(1, kSEpi);
-    if (rv)
-      for (int l = part; l < 16; l += kParts) {
-        float4 a = reinterpret_cast<float4*>(g.gT)[(long)l * rows + row];
+    if (rv) {
+      float4 a[16 / kParts];
+#pragma unroll
+      for (int i = 0; i < 16 / kParts; ++i)
+        a[i] = reinterpret_cast<float4*>(g.gT)[(long)(part + kParts * i) * rows + row];
+#pragma unroll
+      for (int i = 0; i < 16 / kParts; ++i) {
+        const int l = part + kParts * i;
+#pragma unroll
         for (int pp = 0; pp < kParts; ++pp) {
-          const float4 e = *reinterpret_cast<const float4*>(s_ext + ((pp * SBM) + rl) * 64 + l * 4);
-          a.x += e.x;
-          a.y += e.y;
-          a.z += e.z;
-          a.w += e.w;
+          const float4 e = *reinterpret_cast<const float4*>(s_ext + ((pp * SBM) + rl) * 68 + l * 4);
+          a[i].x += e.x;
+          a[i].y += e.y;
+          a[i].z += e.z;
+          a[i].w += e.w;
         }
-        reinterpret_cast<float4*>(g.gT)[(long)l * rows + row] = a;
+        reinterpret_cast<float4*>(g.gT)[(long)l * rows + row] = a[i];
       }
+    }
   }
   }
   tc_fence_before();
@@ -537,10 +648,9 @@ __global__ void __launch_bounds__(kSThreads, 1) k_fit_split(const __grid_constan
   if (warp == kProd) tmem_dealloc(tmem, 512);
 }
 
-// ring, barriers, then either the forward's energies, biases and output weights or (dE/dT mode) T_< rows
-size_t split_smem() {
-  const size_t tail = std::max<size_t>((kParts * SBM + kSL * 256 + 256) * 4, (size_t)SBM * 16 * 16);
-  return (size_t)kSRing * kSStage + 16 * 8 + 16 + tail + 1024;
+// the buffer, barriers, energies, biases and output weights
+size_t split_smem(int rows) {
+  return (size_t)buffer_bytes(rows) + (2 * kP0 + 6 + 2 + 2 + 4 + 1 + 2 * kCRing + 1) * 8 + 16 + (kParts * SBM + kSL * 256 + 256) * 4 + 1024;
 }
 
 }  // namespace
@@ -568,8 +678,9 @@ int run_fitting_split(const DeviceModel& m, const PathConst& pc, const __nv_bflo
   const int nt = pc.ntypes;
   const int KD = pc.M * pc.A;
   const bool gtm = gT != nullptr && Tm != nullptr && pc.A == 16;
-  __nv_bfloat16* xs = ar.get<__nv_bfloat16>(4 * N * kSLd);
-  float* gate = ar.get<float>((long)nh * N * kSLd);
+  const long max_tiles = (N + SBM - 1) / SBM + nt;  // every type's last tile may be short
+  float* resid = ar.get<float>(max_tiles * SBM * kSLd);
+  float* gate = ar.get<float>((long)nh * max_tiles * SBM * kSLd);
   float* gD = gtm ? nullptr : ar.get<float>(N * KD);
   if (ar.measure) return DP_OK;
   if (!ar.ok()) {
@@ -585,6 +696,9 @@ int run_fitting_split(const DeviceModel& m, const PathConst& pc, const __nv_bflo
     a.width[l + 1] = m.fit[l].n_out;
     a.skip[l] = m.fit[l].skip;
   }
+  int maxw = 0;
+  for (int l = 0; l < nh; ++l) maxw = std::max(maxw, a.width[l + 1]);
+  a.rows = slot_rows(maxw);
   int tiles = 0;
   for (int t = 0; t <= nt; ++t) {
     a.row_start[t] = io.type_start[t];
@@ -593,18 +707,8 @@ int run_fitting_split(const DeviceModel& m, const PathConst& pc, const __nv_bflo
   }
   SplitMaps mp;
   std::memset(&mp, 0, sizeof(mp));
-  int rc = make_tmap_bf16(&mp.d[0], Dhi, N, KD, SBM);
-  if (rc == DP_OK) rc = make_tmap_bf16(&mp.d[1], Dlo, N, KD, SBM);
-  for (int b = 0; rc == DP_OK && b < 2; ++b)
-    for (int hl = 0; rc == DP_OK && hl < 2; ++hl) {
-      a.xs[b][hl] = xs + (long)(2 * b + hl) * N * kSLd;
-      rc = make_tmap_bf16(&mp.x[b][hl], a.xs[b][hl], N, kSLd, SBM);
-      for (int t = 0; rc == DP_OK && t < nt; ++t) {
-        const long n_t = io.type_start[t + 1] - io.type_start[t];
-        if (n_t > 0)
-          rc = make_tmap_bf16(&mp.xt[t][b][hl], a.xs[b][hl] + (long)io.type_start[t] * kSLd, n_t, kSLd, SBM);
-      }
-    }
+  int rc = make_tmap_bf16(&mp.d[0], Dhi, N, KD, SBM, kKB);
+  if (rc == DP_OK) rc = make_tmap_bf16(&mp.d[1], Dlo, N, KD, SBM, kKB);
   if (rc != DP_OK) return rc;
   const float* p32 = m.p32;
   for (int t = 0; t < nt; ++t) {
@@ -612,8 +716,8 @@ int run_fitting_split(const DeviceModel& m, const PathConst& pc, const __nv_bflo
       const LayerDesc& L = m.fit[(size_t)t * nfl + l];
       a.bias[t][l] = p32 + L.w_off + (long)L.n_in * L.n_out;
       for (int hl = 0; hl < 2; ++hl) {
-        const CUtensorMap* f = fit_weight_map(m, t, l, 0, L.n_out, hl == 1);
-        const CUtensorMap* b = fit_weight_map(m, t, l, 1, l == 0 ? 256 : L.n_in, hl == 1);
+        const CUtensorMap* f = fit_weight_map(m, t, l, 0, L.n_out, hl == 1, kKB);
+        const CUtensorMap* b = l == 0 ? fit_weight_map(m, t, 0, 1, CH, hl == 1, kKB) : fit_weight_map(m, t, l, 1, L.n_in, hl == 1, kKB);
         if (!f || !b) return DP_E_CUDA;
         mp.w[t][l][hl] = *f;
         mp.w[t][nh + l][hl] = *b;
@@ -623,6 +727,7 @@ int run_fitting_split(const DeviceModel& m, const PathConst& pc, const __nv_bflo
     a.w_last[t] = p32 + Lo.w_off;
     a.b_last[t] = m.fit_out_bias[t];
   }
+  a.resid = resid;
   a.gate = gate;
   a.perm = io.perm;
   a.atom_e = io.atom_energy;
@@ -633,7 +738,7 @@ int run_fitting_split(const DeviceModel& m, const PathConst& pc, const __nv_bflo
   a.err = &io.status->timeout;
   if (tiles > 0) {
     ProfScope _ps(io.prof, "fit_split_tc", st);
-    const size_t smem = split_smem();
+    const size_t smem = split_smem(a.rows);
     DP_CUDA_TRY(allow_max_smem(k_fit_split));
     k_fit_split<<<tiles, kSThreads, smem, st>>>(mp, a);
     DP_CUDA_TRY(cudaGetLastError());

@@ -34,8 +34,8 @@ int skip_kind(int n_in, int n_out) { return n_out == n_in ? 1 : (n_out == 2 * n_
 
 // Tensor map of fitting layer l of type t: dir 0 the forward B operand W^T [n_out][n_in], dir 1
 // the backward one W [n_in][n_out]; box of 64 columns x box_rows rows; cached on the model.
-const CUtensorMap* fit_weight_map(const DeviceModel& m, int t, int l, int dir, int box_rows, bool lo) {
-  const long key = ((((long)t * 64 + l) * 2 + dir) * 1024 + box_rows) * 2 + (lo ? 1 : 0);
+const CUtensorMap* fit_weight_map(const DeviceModel& m, int t, int l, int dir, int box_rows, bool lo, int box_cols) {
+  const long key = (((((long)t * 64 + l) * 2 + dir) * 1024 + box_rows) * 2 + (lo ? 1 : 0)) * 2 + (box_cols == 64 ? 0 : 1);
   for (auto& kv : m.tmap_cache)
     if (kv.first == key) return reinterpret_cast<const CUtensorMap*>(kv.second.data());
   const int nfl = m.n_fit_layers;
@@ -51,9 +51,9 @@ const CUtensorMap* fit_weight_map(const DeviceModel& m, int t, int l, int dir, i
     return nullptr;
   }
   if (dir == 0)  // forward B^T = W^T [n_out][n_in]
-    rc = make_tmap_bf16(map, static_cast<const __nv_bfloat16*>(wt) + off, L.n_out, L.n_in, box_rows);
+    rc = make_tmap_bf16(map, static_cast<const __nv_bfloat16*>(wt) + off, L.n_out, L.n_in, box_rows, box_cols);
   else  // backward B^T = W [n_in][n_out]
-    rc = make_tmap_bf16(map, static_cast<const __nv_bfloat16*>(w) + off, L.n_in, L.n_out, box_rows);
+    rc = make_tmap_bf16(map, static_cast<const __nv_bfloat16*>(w) + off, L.n_in, L.n_out, box_rows, box_cols);
   if (rc != DP_OK) return nullptr;
   m.tmap_cache.emplace_back(key, std::move(buf));
   return reinterpret_cast<const CUtensorMap*>(m.tmap_cache.back().second.data());

@@ -16,9 +16,10 @@ bool fit_tc_supported(const DeviceModel& m);
 
 // Energies (and their FP64 sum) and dE/dD [N][M*M_<] (FP32) from the BF16 descriptor.
 // Tensor map of fitting layer l of type t (dir 0: W^T [n_out][n_in], dir 1: W [n_in][n_out]),
-// box of 64 columns x box_rows rows, cached on the model.
+// box of box_cols columns (64, or 32 with 64-byte swizzle) x box_rows rows, cached on the model.
 // lo selects the low halves (split operands).
-const CUtensorMap* fit_weight_map(const DeviceModel& m, int t, int l, int dir, int box_rows, bool lo = false);
+const CUtensorMap* fit_weight_map(const DeviceModel& m, int t, int l, int dir, int box_rows, bool lo = false,
+                                  int box_cols = 64);
 // The whole fitting net (forward to E_i, backward to dE/dD in BF16) in one kernel per 128-atom
 // tile, for nets of at most four hidden layers of width <= 256 (multiples of 16) with skips of
 // kind 0 or 1.

@@ -336,7 +336,7 @@ std::mutex g_encode_mu;
 
 }  // namespace
 
-int make_tmap_bf16(CUtensorMap* map, const void* base, long rows, long cols, int box_rows) {
+int make_tmap_bf16(CUtensorMap* map, const void* base, long rows, long cols, int box_rows, int box_cols) {
   {
     std::lock_guard<std::mutex> lk(g_encode_mu);
     if (!g_encode) {
@@ -350,16 +350,18 @@ int make_tmap_bf16(CUtensorMap* map, const void* base, long rows, long cols, int
       g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
     }
   }
-  if ((cols * 2) % 16 != 0 || (reinterpret_cast<uintptr_t>(base) & 15) != 0 || box_rows < 1 || box_rows > 256) {
+  if ((cols * 2) % 16 != 0 || (reinterpret_cast<uintptr_t>(base) & 15) != 0 || box_rows < 1 || box_rows > 256 ||
+      (box_cols != BK && box_cols != BK / 2)) {
     set_error("tensor map: row pitch and base must be 16-byte aligned, box rows in [1, 256]");
     return DP_E_UNSUPPORTED;
   }
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)(cols * 2)};
-  cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
+  cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        box_cols == BK ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     set_error("cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");

@@ -113,6 +113,17 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
   return d;
 }
 
+// The same with 64-byte swizzle: rows of 64 bytes, 8-row groups 512 bytes apart.
+__device__ __forceinline__ uint64_t sdesc_sw64(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(512 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;            // 64-byte swizzle
+  return d;
+}
+
 // Instruction descriptor of kind::f16 with FP32 accumulation, both operands K-major.
 // bf16 = 1 selects BF16 operands, 0 FP16 (A and B always have the same type).
 __host__ __device__ constexpr uint32_t idesc_f16(int m, int n, int bf16) {
@@ -125,6 +136,32 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t ad, uint64_t bd,
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
           tmem),
       "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+      : "memory");
+}
+// One lane of a converged warp (the same one every time), as a 0 / 1 value for the _by forms below.
+__device__ __forceinline__ uint32_t elect_lane() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e;
+}
+// mma_f16 issued by the lane whose `by` is 1, in code the whole warp runs, so that its operands are warp
+// uniform to the compiler.
+__device__ __forceinline__ void mma_f16_by(uint32_t by, uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc,
+                                           uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+      "l"(ad), "l"(bd), "r"(idesc), "r"(acc), "r"(by)
+      : "memory");
+}
+// The same with the A operand in tensor memory: row = lane, 32-bit column j holds elements 2j and 2j + 1
+// of the row, so 16 elements of K are eight columns.
+__device__ __forceinline__ void mma_f16_ta_by(uint32_t by, uint32_t tmem, uint32_t a, uint64_t bd, uint32_t idesc,
+                                              uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem),
+      "r"(a), "l"(bd), "r"(idesc), "r"(acc), "r"(by)
       : "memory");
 }
 // Instruction descriptor of kind::tf32 (TF32 operands read from FP32 storage, FP32 accumulation),
@@ -144,6 +181,14 @@ __device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t ad, uint64_t bd
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(bar))
                : "memory");
+}
+
+__device__ __forceinline__ void mma_commit_by(uint32_t by, uint64_t* bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(su32(bar)),
+      "r"(by)
+      : "memory");
 }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t* holder, uint32_t ncols) {
@@ -179,6 +224,12 @@ __device__ __forceinline__ void tmem_st16(uint32_t addr, const float* v) {
       "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])),
       "r"(__float_as_uint(v[15]))
       : "memory");
+}
+// Eight 32-bit columns (16 BF16 values) of each of the warp's 32 TMEM lanes.
+__device__ __forceinline__ void tmem_st8(uint32_t addr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
