@@ -231,6 +231,7 @@ struct NlLaunch {
   int nframes;            // frames in the launch
   int max_noff;           // largest (2K_0+1)(2K_1+1)(2K_2+1) over the frames
   int max_stream;         // largest mean candidate stream of one cell over the frames (0: unknown)
+  bool pdl = false;       // programmatic dependent launches (pdl.cuh)
   double max_cell_atoms = 0.0;  // largest mean number of atoms of a cell over the frames (0: unknown)
 };
 // What a path call also takes from the list build: the (type, cell) order of the atoms as its

@@ -13,6 +13,7 @@
 
 #include "capi_internal.cuh"
 #include "grad.cuh"
+#include "pdl.cuh"
 #include "table.cuh"
 
 namespace dpgb {
@@ -56,6 +57,8 @@ __global__ void __launch_bounds__(320)
                  double* __restrict__ cpart, const int* __restrict__ frame_chunk, int nframes, int* __restrict__ fcount,
                  double* __restrict__ energy, double* __restrict__ virial) {
   __shared__ int s_last;
+  pdl_wait();
+  pdl_next();
   const int c = blockIdx.x, lane = threadIdx.x & 31, q = threadIdx.x >> 5;  // component q
   // the sum over n rows of one component, rows s apart
   auto sum_rows = [&](const double* v, long s, int n) {
@@ -104,6 +107,7 @@ struct ClearArgs {
   long n[5];  // 32-bit words
 };
 __global__ void k_clear(const ClearArgs a) {
+  pdl_next();
   const long t = (long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long)gridDim.x * blockDim.x;
 #pragma unroll
   for (int k = 0; k < 5; ++k)
@@ -412,6 +416,9 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
   // All device work of the call, in stream order on s (tables uploaded from `stage`); the
   // path's scratch is carved afresh from the same arena position every time.
   const size_t ar_used0 = ar.used;
+  // small frames of the moment path: programmatic dependent launches (not while kernels are being timed)
+  const bool pdl = N <= kPdlAtoms && !gr && own_nlist && !md->prof.timing && m.compressed &&
+                   m.cfg.descriptor == DP_DESC_SE_E2_A && m.mom_npass != 0;
   auto enqueue = [&](cudaStream_t s, unsigned char* stage) -> int {
     ar.used = ar_used0;
     ar.fail = false;
@@ -456,7 +463,7 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
       // the list build's (type, cell) order is the path's type-sorted order, and its first
       // launch also forms the image translations
       NlLaunch L{N, T.ncells, T.cap, d_geoms, b.atom_frame, F > 1 ? d_celloff : nullptr, F, T.max_noff(),
-                 T.max_stream(), T.max_cell_atoms()};
+                 T.max_stream(), pdl, T.max_cell_atoms()};
       // the moment path reads its list in batches
       const bool lean = m.compressed && m.cfg.descriptor == DP_DESC_SE_E2_A && m.mom_npass != 0;
       NlExtras ex{b.perm, b.type_start, chk, d_boxes, T.periodic ? F : 0, T.periodic ? b.tshift : nullptr, b.disp,
@@ -490,6 +497,7 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
       }
     }
     io.prof = &md->prof;
+    io.pdl = pdl;
     io.coord = dcoord;
     io.type = dtype;
     io.perm = b.perm;
@@ -519,8 +527,8 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
     double* d_virial = host_v ? b.virial : virial;
     {
       ProfScope _ps(&md->prof, "frame_sums", s);
-      k_chunk_sums<<<T.C, 320, 0, s>>>(d_chunk, io.atom_energy, io.atom_virial, b.cpart, d_fchunk, F, b.fcount,
-                                          d_energy, d_virial);
+      DP_CUDA_TRY(launch_chain(pdl, k_chunk_sums, dim3(T.C), dim3(320), 0, s, d_chunk, io.atom_energy, io.atom_virial,
+                               b.cpart, d_fchunk, F, b.fcount, d_energy, d_virial));
     }
     DP_CUDA_TRY(cudaGetLastError());
     if (host_e) DP_CUDA_TRY(cudaMemcpyAsync(energy, d_energy, sizeof(double) * F, cudaMemcpyDeviceToHost, s));
@@ -772,7 +780,7 @@ int dp_build_nlist(dp_model* md, int N, const double* coord, const int* type, co
   DP_CUDA_TRY(cudaMemsetAsync(md->status, 0, sizeof(DevStatus), st));
   {
     NlLaunch L{N, T.ncells, T.cap, reinterpret_cast<const NlGeom*>(b.ftab + T.off_geoms), nullptr, nullptr, 1,
-               T.max_noff(), T.max_stream(), T.max_cell_atoms()};
+               T.max_noff(), T.max_stream(), false, T.max_cell_atoms()};
     ProfScope _ps(&md->prof, "nlist", st, nlist_launches(L, m.cfg.ntypes));
     const NlScratch sc{b.cell_count, b.cell_start, b.atom_key, b.atom_l, b.atom_m, b.sorted_l, b.sorted_m};
     DP_CUDA_TRY(launch_nlist_build(L, m.cfg.ntypes, dcoord, dtype, sc, nl->nl_j, nl->nl_code, nl->counts, md->status,

@@ -172,6 +172,7 @@ int run_fitting_tc(const DeviceModel& m, const PathConst& pc, const __nv_bfloat1
   TcArgs base;
   std::memset(&base, 0, sizeof(base));
   base.ntypes = nt;
+  base.pdl = io.pdl;
   int tiles = 0;
   for (int t = 0; t <= nt; ++t) {
     base.row_start[t] = io.type_start[t];
@@ -248,7 +249,7 @@ int run_fitting_tc(const DeviceModel& m, const PathConst& pc, const __nv_bfloat1
   {
     ProfScope _ps(io.prof, "energy_sum", st);
     const int bn = pick_bn(m.fit[nh - 1].n_out, true);
-    DP_CUDA_TRY(launch_energy_f32(E, (m.fit[nh - 1].n_out + bn - 1) / bn, io.perm, (int)N, io.atom_energy, st));
+    DP_CUDA_TRY(launch_energy_f32(E, (m.fit[nh - 1].n_out + bn - 1) / bn, io.perm, (int)N, io.atom_energy, st, io.pdl));
   }
   // ---- backward ----
   for (int l = nh - 1; l >= 0; --l) {

@@ -42,6 +42,7 @@
 #include "env.cuh"
 #include "fit_tc.cuh"
 #include "mom.cuh"
+#include "pdl.cuh"
 #include "tc_gemm.cuh"
 #include "tc_ptx.cuh"
 
@@ -264,6 +265,8 @@ __global__ void __launch_bounds__(256, 3)
     k_env_mom(PathConst pc, MomArgs g, const double* __restrict__ coord, const int* __restrict__ nl_code) {
   constexpr int PARTS = NPASS == 1 ? 1 : 2;
   __shared__ float s_carry[8][24];  // moments of the run left open at a batch's end, per warp
+  pdl_wait();
+  pdl_next();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* carry = s_carry[warp];
   const long ntask = (long)pc.natoms * pc.ntypes;
@@ -524,6 +527,8 @@ __global__ void __launch_bounds__(kMomThreads, NPASS == 1 ? 3 : 1)
     mbar_fence_init();
   }
   if (warp == 4) tmem_alloc(tmem_holder, 128);
+  pdl_wait();
+  pdl_next();
   const int r = threadIdx.x;
   const int ae = r >> 2, c = r & 3;
   const int pe = row0 + ae;
@@ -761,6 +766,8 @@ __global__ void __launch_bounds__(kRows)
   constexpr int SCRP = NPAD + 4;  // FP32 scratch row pitch
   __shared__ __align__(16) float scr[16 * SCRP];
   static_assert(NGRP == 8, "eight groups of four atoms per tile");
+  pdl_wait();
+  pdl_next();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, c = lane & 3;
   int ti = 0;
   while (ti + 1 < g.ntypes && (int)blockIdx.x >= g.tile_start[ti + 1]) ++ti;
@@ -934,6 +941,8 @@ __global__ void __launch_bounds__(kMomThreads, 1)
     mbar_fence_init();
   }
   if (warp == 4) tmem_alloc(tmem_holder, 64 * kAccBufs);
+  pdl_wait();
+  pdl_next();
   const int r = threadIdx.x;
   const int ae = r >> 2, c = r & 3;
   const int pe = row0 + ae;
@@ -1122,6 +1131,8 @@ __global__ void __launch_bounds__(kMomThreads, 1)
 // =============================================================================================
 __global__ void __launch_bounds__(256)
     k_force_mom(PathConst pc, MomArgs g) {
+  pdl_wait();
+  pdl_next();
   const int p = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (p >= pc.natoms) return;  // warp-uniform
@@ -1268,30 +1279,30 @@ size_t bwd_smem(int npass, int nc) {
 }
 
 template <int NPASS, int NPAD>
-int launch_mom(const DeviceModel& m, const MomArgs& g, int tiles, int which, cudaStream_t st) {
+int launch_mom(const DeviceModel& m, const MomArgs& g, int tiles, int which, bool pdl, cudaStream_t st) {
   const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(m.mom_maps.data());
   if (which == 1) {
-    k_mom_gT<NPASS, NPAD><<<dim3(tiles, kAtoms / kGroupAtoms), kRows, 0, st>>>(g);
+    DP_CUDA_TRY(launch_chain(pdl, k_mom_gT<NPASS, NPAD>, dim3(tiles, kAtoms / kGroupAtoms), dim3(kRows), 0, st, g));
   } else if (which == 0) {
     const size_t sm = fwd_smem(NPASS, NPAD, g.nc);
     DP_CUDA_TRY(allow_max_smem(k_mom_fwd<NPASS, NPAD>));
-    k_mom_fwd<NPASS, NPAD><<<tiles, kMomThreads, sm, st>>>(maps[0], maps[1], g);
+    DP_CUDA_TRY(launch_chain(pdl, k_mom_fwd<NPASS, NPAD>, dim3(tiles), dim3(kMomThreads), sm, st, maps[0], maps[1], g));
   } else {
     const size_t sm = bwd_smem(NPASS, g.nc);
     DP_CUDA_TRY(allow_max_smem(k_mom_bwd<NPASS, NPAD>));
-    k_mom_bwd<NPASS, NPAD><<<tiles, kMomThreads, sm, st>>>(maps[2], maps[3], g);
+    DP_CUDA_TRY(launch_chain(pdl, k_mom_bwd<NPASS, NPAD>, dim3(tiles), dim3(kMomThreads), sm, st, maps[2], maps[3], g));
   }
   DP_CUDA_TRY(cudaGetLastError());
   return DP_OK;
 }
 
 template <int NPASS>
-int launch_mom_np(const DeviceModel& m, const MomArgs& g, int tiles, int which, cudaStream_t st) {
-  if (m.mom_npad == 16) return launch_mom<NPASS, 16>(m, g, tiles, which, st);
-  if (m.mom_npad == 32) return launch_mom<NPASS, 32>(m, g, tiles, which, st);
-  if (m.mom_npad == 64) return launch_mom<NPASS, 64>(m, g, tiles, which, st);
-  if (m.mom_npad == 112) return launch_mom<NPASS, 112>(m, g, tiles, which, st);
-  if (m.mom_npad == 128) return launch_mom<NPASS, 128>(m, g, tiles, which, st);
+int launch_mom_np(const DeviceModel& m, const MomArgs& g, int tiles, int which, bool pdl, cudaStream_t st) {
+  if (m.mom_npad == 16) return launch_mom<NPASS, 16>(m, g, tiles, which, pdl, st);
+  if (m.mom_npad == 32) return launch_mom<NPASS, 32>(m, g, tiles, which, pdl, st);
+  if (m.mom_npad == 64) return launch_mom<NPASS, 64>(m, g, tiles, which, pdl, st);
+  if (m.mom_npad == 112) return launch_mom<NPASS, 112>(m, g, tiles, which, pdl, st);
+  if (m.mom_npad == 128) return launch_mom<NPASS, 128>(m, g, tiles, which, pdl, st);
   set_error("moment path: unsupported padded width");
   return DP_E_UNSUPPORTED;
 }
@@ -1445,15 +1456,13 @@ int run_mom(const DeviceModel& m, const PathConst& pc, const PathIO& io, Arena& 
     // one warp per (atom, neighbour type) task; persistent warps, three 8-warp blocks per SM
     const long tasks = N * pc.ntypes;
     const unsigned blocks = (unsigned)std::min<long>((tasks + 7) / 8, 3L * sm_count());
-    if (bf16)
-      k_env_mom<1><<<blocks, 256, 0, st>>>(pc, g, io.coord, io.nl_code);
-    else
-      k_env_mom<3><<<blocks, 256, 0, st>>>(pc, g, io.coord, io.nl_code);
-    DP_CUDA_TRY(cudaGetLastError());
+    DP_CUDA_TRY(launch_chain(io.pdl, bf16 ? k_env_mom<1> : k_env_mom<3>, dim3(blocks), dim3(256), 0, st, pc, g, io.coord,
+                             io.nl_code));
   }
   if (tiles > 0) {
     ProfScope _ps(io.prof, "mom_fwd", st);
-    const int rc = bf16 ? launch_mom_np<1>(m, g, tiles, 0, st) : launch_mom_np<3>(m, g, tiles, 0, st);
+    const int rc = bf16 ? launch_mom_np<1>(m, g, tiles, 0, io.pdl, st)
+                        : launch_mom_np<3>(m, g, tiles, 0, io.pdl, st);
     if (rc != DP_OK) return rc;
   }
   int rc;
@@ -1470,17 +1479,16 @@ int run_mom(const DeviceModel& m, const PathConst& pc, const PathIO& io, Arena& 
   if (tiles > 0) {
     if (!g.gTt) {
       ProfScope _ps(io.prof, "mom_gT", st);
-      rc = bf16 ? launch_mom_np<1>(m, g, tiles, 1, st) : launch_mom_np<3>(m, g, tiles, 1, st);
+      rc = bf16 ? launch_mom_np<1>(m, g, tiles, 1, io.pdl, st) : launch_mom_np<3>(m, g, tiles, 1, io.pdl, st);
       if (rc != DP_OK) return rc;
     }
     {
       ProfScope _ps(io.prof, "mom_bwd", st);
-      rc = bf16 ? launch_mom_np<1>(m, g, tiles, 2, st) : launch_mom_np<3>(m, g, tiles, 2, st);
+      rc = bf16 ? launch_mom_np<1>(m, g, tiles, 2, io.pdl, st) : launch_mom_np<3>(m, g, tiles, 2, io.pdl, st);
       if (rc != DP_OK) return rc;
     }
     ProfScope _ps(io.prof, "mom_force", st);
-    k_force_mom<<<(unsigned)((N * 32 + 255) / 256), 256, 0, st>>>(pc, g);
-    DP_CUDA_TRY(cudaGetLastError());
+    DP_CUDA_TRY(launch_chain(io.pdl, k_force_mom, dim3((unsigned)((N * 32 + 255) / 256)), dim3(256), 0, st, pc, g));
   }
   return DP_OK;
 }

@@ -17,6 +17,7 @@
 #include <cstdio>
 
 #include "dp_internal.cuh"
+#include "pdl.cuh"
 
 namespace dpgb {
 
@@ -98,6 +99,8 @@ __global__ void k_bin(const NlGeom* __restrict__ G, const int* __restrict__ atom
                       int2* __restrict__ atom_key, float4* __restrict__ atom_l, int4* __restrict__ atom_m,
                       DevStatus* __restrict__ st, const double* __restrict__ boxes, int nframes,
                       double* __restrict__ tshift) {
+  pdl_wait();
+  pdl_next();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (tshift)
     for (int k = i; k < 27 * nframes; k += gridDim.x * blockDim.x) {
@@ -212,6 +215,8 @@ __global__ void k_fill_scan(int natoms, const int* __restrict__ cell_count, int 
                             int* __restrict__ perm, int* __restrict__ type_start, int ncells_total, int ntypes,
                             DevStatus* __restrict__ st, const TypeStartCheck chk) {
   extern __shared__ int s_start[];  // [nkeys + 1]
+  pdl_wait();
+  pdl_next();
   block_scan_counts(cell_count, nkeys, s_start);
   if (blockIdx.x == 0)
     for (int k = threadIdx.x; k <= nkeys; k += blockDim.x) cell_start[k] = s_start[k];
@@ -655,6 +660,8 @@ __global__ void __launch_bounds__(kCellWarps * 32, CAP <= 256 ? 4 : 3)
   unsigned* hist = reinterpret_cast<unsigned*>(e_key + CAPP);  // two 16-bit counters a word; then bucket ends
   unsigned short* e_ref = reinterpret_cast<unsigned short*>(hist + NB / 2);
 
+  pdl_wait();
+  pdl_next();
   const int gc = blockIdx.x;  // cell, all frames
   // this block's share of the cell's centre atoms: per_block of them from blockIdx.y * per_block on
   // (and again every gridDim.y * per_block where the cell holds more than expected)
@@ -1306,15 +1313,22 @@ cudaError_t launch_nlist_build(const NlLaunch& L, int ntypes, const double* coor
   const int bin_threads = 64;
   TypeStartCheck nochk;
   std::memset(&nochk, 0, sizeof(nochk));
-  k_bin<<<(L.natoms + bin_threads - 1) / bin_threads, bin_threads, 0, st>>>(L.geoms, L.atom_frame, L.cell_off, L.natoms, L.ncells_total, ntypes, coord, type,
-                            cell_count, sc.atom_key, sc.atom_l, sc.atom_m, status, ex ? ex->boxes : nullptr,
-                            ex ? ex->nframes : 0, ex ? ex->tshift : nullptr);
+  const double* no_boxes = nullptr;
+  double* no_tshift = nullptr;
+  e = launch_chain(L.pdl, k_bin, dim3((L.natoms + bin_threads - 1) / bin_threads), dim3(bin_threads), 0, st, L.geoms,
+                   L.atom_frame, L.cell_off, L.natoms, L.ncells_total, ntypes, coord, type, cell_count, sc.atom_key,
+                   sc.atom_l, sc.atom_m, status, ex ? ex->boxes : no_boxes, ex ? ex->nframes : 0,
+                   ex ? ex->tshift : no_tshift);
+  if (e != cudaSuccess) return e;
+  int* no_int = nullptr;
   if (nkeys <= 8192) {  // few keys: each fill block scans the counts itself (one launch fewer; nlist_launches)
     // wider blocks for many keys: each thread scans up to eight of them
     const int ft = nkeys <= 2048 ? 256 : 1024;
-    k_fill_scan<<<(L.natoms + ft - 1) / ft, ft, (size_t)(nkeys + 1) * sizeof(int), st>>>(
-        L.natoms, cell_count, nkeys, cell_start, sc.atom_key, sc.atom_l, sc.atom_m, sc.sorted_l, sc.sorted_m,
-        ex ? ex->perm : nullptr, ex ? ex->type_start : nullptr, L.ncells_total, ntypes, status, ex ? ex->chk : nochk);
+    e = launch_chain(L.pdl, k_fill_scan, dim3((L.natoms + ft - 1) / ft), dim3(ft), (size_t)(nkeys + 1) * sizeof(int), st,
+                     L.natoms, cell_count, nkeys, cell_start, sc.atom_key, sc.atom_l, sc.atom_m, sc.sorted_l, sc.sorted_m,
+                     ex ? ex->perm : no_int, ex ? ex->type_start : no_int, L.ncells_total, ntypes, status,
+                     ex ? ex->chk : nochk);
+    if (e != cudaSuccess) return e;
   } else {
     k_scan_excl<<<1, 1024, 0, st>>>(cell_count, nkeys, cell_start, nullptr);
     k_fill<<<nb, 256, 0, st>>>(L.natoms, sc.atom_key, sc.atom_l, sc.atom_m, sc.sorted_l, sc.sorted_m,
@@ -1331,6 +1345,7 @@ cudaError_t launch_nlist_build(const NlLaunch& L, int ntypes, const double* coor
   const int S = std::max(1024, ((int)(1.25 * mean_stream) + 64 * ntypes + 64 + 127) & ~127);
   const size_t csm = cell_smem_bytes(ccap, S);
   if (L.max_noff > 0 && (long)L.max_noff * ntypes <= kMaxRanges && ccap <= 512 && csm <= 160 * 1024 && S < 65536) {
+    float4* no_disp = nullptr;
     // Centre atoms per block: one a warp (8) or two (16) when the grid then still fits the chip at once
     // (192 atoms: 37 -> 17 us), else a whole cell, up to three a warp (a cell of a box barely wider than r_c
     // holds hundreds of atoms, and one block for all of them left the rest of the chip waiting).
@@ -1344,9 +1359,10 @@ cudaError_t launch_nlist_build(const NlLaunch& L, int ntypes, const double* coor
   do {                                                                                                           \
     e = allow_max_smem(k_nlist_cell<C>);                                                                         \
     if (e != cudaSuccess) return e;                                                                              \
-    k_nlist_cell<C><<<dim3(L.ncells_total, parts), kCellWarps * 32, csm, st>>>(                                  \
-        L.geoms, L.cell_off, L.nframes, L.ncells_total, ntypes, coord, cell_start, sorted_l, sorted_m, S, nl_j,    \
-        nl_code, counts, ex ? ex->disp : nullptr, per_block, ex && ex->lean, status);                            \
+    e = launch_chain(L.pdl, k_nlist_cell<C>, dim3(L.ncells_total, parts), dim3(kCellWarps * 32), csm, st, L.geoms,   \
+                     L.cell_off, L.nframes, L.ncells_total, ntypes, coord, cell_start, sorted_l, sorted_m, S, nl_j, \
+                     nl_code, counts, ex ? ex->disp : no_disp, per_block, ex && ex->lean, status);               \
+    if (e != cudaSuccess) return e;                                                                              \
   } while (0)
     if (ccap <= 128)
       DPGB_NLC_LAUNCH(128);

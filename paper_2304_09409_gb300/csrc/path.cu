@@ -22,6 +22,7 @@
 #include "dp_internal.cuh"
 #include "path.cuh"
 #include "env.cuh"
+#include "pdl.cuh"
 #include "tabeval.cuh"
 
 namespace dpgb {
@@ -868,6 +869,8 @@ __global__ void k_sum_rows(const double* __restrict__ in, long n, int w, double*
 // a fixed order and scattered to input order in FP64.
 __global__ void k_energy_parts(const float* __restrict__ parts, int nparts, const int* __restrict__ perm, int n,
                                double* __restrict__ atom_e) {
+  pdl_wait();
+  pdl_next();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   float e = parts[p];
@@ -1386,9 +1389,8 @@ int run_generic(const DeviceModel& m, const PathConst& pc, const R* params, cons
 }
 
 cudaError_t launch_energy_f32(const float* Eparts, int nparts, const int* perm, int n, double* atom_e,
-                              cudaStream_t st) {
-  k_energy_parts<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(Eparts, nparts, perm, n, atom_e);
-  return cudaGetLastError();
+                              cudaStream_t st, bool pdl) {
+  return launch_chain(pdl, k_energy_parts, dim3((n + 255) / 256), dim3(256), 0, st, Eparts, nparts, perm, n, atom_e);
 }
 
 cudaError_t launch_shift_table(const PathConst& pc, double* out, cudaStream_t st) {

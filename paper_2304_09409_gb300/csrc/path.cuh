@@ -160,6 +160,7 @@ struct ProfScope {
 
 struct PathIO {
   Prof* prof;  // may be null
+  bool pdl;    // programmatic dependent launches along the moment path (pdl.cuh)
   const double* coord;  // device [N][3]
   const int* type;      // device [N]
   const int* perm;      // device [N] sorted position -> atom
@@ -241,7 +242,7 @@ cudaError_t launch_sum_rows(const double* in, long n, int w, double* out, cudaSt
 // Per-atom energies given as nparts FP32 partial sums [nparts][n] (sorted order), summed in a
 // fixed order, to input order in FP64.
 cudaError_t launch_energy_f32(const float* Eparts, int nparts, const int* perm, int n, double* atom_e,
-                              cudaStream_t st);
+                              cudaStream_t st, bool pdl = false);
 // t(n) for n in {-1,0,1}^3 into out [27][3] (device)
 cudaError_t launch_shift_table(const PathConst& pc, double* out, cudaStream_t st);
 

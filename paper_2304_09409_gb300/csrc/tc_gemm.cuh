@@ -25,6 +25,8 @@ struct TcArgs {
   int ntypes;
   int row_start[DP_MAX_TYPES + 1];   // rows of type t: [row_start[t], row_start[t+1])
   int tile_start[DP_MAX_TYPES + 1];  // prefix of 128-row tiles per type
+  bool pdl;                          // programmatic dependent launch (pdl.cuh)
+  int stages;                        // ring stages (set by launch_tc_gemm)
   int K, N, BN;                      // reduction length, output width, output columns per CTA
   const float* bias[DP_MAX_TYPES];   // [N] per type
   const float* w_last[DP_MAX_TYPES];  // FWD_LAST: final linear layer weights [N] per type
