@@ -21,7 +21,6 @@
 
 #include "fit_tc.cuh"
 #include "tc_gemm.cuh"
-#include "pdl.cuh"
 #include "tc_ptx.cuh"
 
 namespace dpgb {

@@ -57,14 +57,13 @@ constexpr int kRows = 128;        // accumulator rows: (atom, c)
 constexpr int kMomThreads = 192;  // 4 builder / epilogue warps, an MMA warp and a TMA producer warp
 constexpr int kABlock = kRows * 128;  // one 64-column K block of 128 rows (bytes)
 constexpr int kGroupAtoms = 4;        // backward: atoms per staged group of dE/dD rows
-// backward: 64-column TMEM accumulators in rotation, and the coefficient ring depth.  The one-pass
-// (mixed) kernel keeps two of each so that three CTAs fit an SM (3 x 128 TMEM columns); the
-// three-pass kernel runs one CTA per SM and takes four accumulators and three stages, so the MMAs
-// of the next chunks run while the epilogue drains one.
+// backward: 64-column TMEM accumulators in rotation.  The one-pass (mixed) kernel keeps two, and two
+// coefficient stages, so that three CTAs fit an SM (3 x 128 TMEM columns); the three-pass kernel runs
+// one CTA per SM and takes four, and four stages where they fit, so the MMAs of the next chunks run
+// while the epilogue drains one.
 template <int NPASS>
 struct BwdDepth {
   static constexpr int acc = NPASS == 1 ? 2 : 4;
-  static constexpr int stages = NPASS == 1 ? 2 : 3;
 };
 
 struct MomArgs {
@@ -80,7 +79,9 @@ struct MomArgs {
   float4* envB;
   int* slot_run;
   // per-run records, run r of type block t of atom p at row p * nc + sel_off[t] + r
-  int* run_l;      // interval of the run; -1 after the last run
+  short* run_l;    // [N][ncl] interval of the run (far below 2^15); -1 after the last run
+  int ncl;         // nc rounded up to 8: rows of run_l are 16-byte aligned
+  uint2* run_mask; // [N][ntypes] bit l >> 2 of every run's interval, or null
   uint4* run_rec;  // moments as A-operand chunks [row][4 components][parts]
   float4* run_P;   // P of the run [row][4 components][2] FP32, or [row][4 components] 8 x BF16 when
                    // p_bf16 (mixed mode); shares memory with run_rec
@@ -133,16 +134,37 @@ __device__ __forceinline__ int mom_interval(const MomArgs& g, float s, int lcap,
   return l;
 }
 
-// Block kb of the tile's schedule: neighbour types in order, 8-interval groups descending.
-__device__ __forceinline__ void block_of(int kb, const int* ghi, int ntypes, int& t, int& grp) {
+// A tile's schedule of K blocks: neighbour types in order, 8-interval groups descending, and (halves) the
+// lower and the upper four intervals of a group as blocks of their own.  With run masks only the blocks
+// that some atom of the tile has a neighbour in are scheduled (the others would add exact zeros): in
+// water the intervals between the O-H bond and everything else are empty.
+constexpr int kSchedMax = DP_MAX_TYPES * 64;
+struct Sched {
+  int n;                            // blocks
+  int ghi[DP_MAX_TYPES];            // no masks: largest group of each type
+};
+// entries (masks only, kSchedMax of them after the kernel's other shared memory): type << 8 | block, a
+// block being a group or 2 * group + half
+template <bool HALVES>
+__device__ __forceinline__ void block_of(const Sched& sc, const unsigned short* entries, int kb, int ntypes, int& t,
+                                         int& grp, int& h) {
+  if (entries) {
+    const int v = entries[kb], blk = v & 255;
+    t = v >> 8;
+    grp = HALVES ? blk >> 1 : blk;
+    h = HALVES ? blk & 1 : 0;
+    return;
+  }
+  h = HALVES ? kb & 1 : 0;
+  if (HALVES) kb >>= 1;
   t = 0;
   while (t < ntypes) {
-    const int n = ghi[t] + 1;
+    const int n = sc.ghi[t] + 1;
     if (kb < n) break;
     kb -= n;
     ++t;
   }
-  grp = ghi[t] - kb;
+  grp = sc.ghi[t] - kb;
 }
 
 // tau of s on interval l (the list order lowered l below the interval of s by a rounding error).
@@ -184,66 +206,79 @@ __device__ __forceinline__ uint32_t sw_off(int r, int q) {
   return (uint32_t)((r >> 3) * 1024 + (r & 7) * 128 + ((q ^ (r & 7)) << 4));
 }
 
-// The run intervals of the tile's 32 atoms, every type block ([atom][nc], -1 past a tile's end),
-// as 16-bit values (intervals are far below 2^15).  The tile's rows are one contiguous stretch of
-// run_l: 16-byte loads where it is aligned, and each thread's loads all in flight before the first
-// store.
+// Copies the run intervals of the tile's 32 atoms ([atom][ncl], every type block; -1 past a tile's end).
 __device__ __forceinline__ void stage_runs(const MomArgs& g, int row0, int row_end, short* runl_s, int tid,
                                            int nthreads) {
-  const int n = kAtoms * g.nc;
-  const int nv = min(kAtoms, row_end - row0) * g.nc;  // slots of the tile's real atoms
-  const int* src = g.run_l + (long)row0 * g.nc;
-  int done = 0;
-  if ((reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
-    const int n4 = nv >> 2;
-    const int4* s4 = reinterpret_cast<const int4*>(src);
-    short4* d4 = reinterpret_cast<short4*>(runl_s);
-    for (int e0 = tid; e0 < n4; e0 += 8 * nthreads) {
-      int4 v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = e0 + u * nthreads;
-        if (e < n4) v[u] = __ldg(s4 + e);
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = e0 + u * nthreads;
-        if (e < n4) d4[e] = make_short4((short)v[u].x, (short)v[u].y, (short)v[u].z, (short)v[u].w);
-      }
-    }
-    done = 4 * n4;
+  const int n8 = kAtoms * g.ncl / 8, nv = min(kAtoms, row_end - row0) * g.ncl / 8;  // 16-byte pieces
+  const uint4* src = reinterpret_cast<const uint4*>(g.run_l + (long)row0 * g.ncl);
+  uint4* dst = reinterpret_cast<uint4*>(runl_s);
+  for (int e = tid; e < n8; e += nthreads) {
+    if (e < nv)
+      cp_async16(dst + e, src + e);
+    else
+      dst[e] = make_uint4(~0u, ~0u, ~0u, ~0u);
   }
-  for (int e0 = done + tid; e0 < n; e0 += 16 * nthreads) {
-    int v[16];
-#pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int e = e0 + u * nthreads;
-      v[u] = e < nv ? __ldg(src + e) : -1;
-    }
-#pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int e = e0 + u * nthreads;
-      if (e < n) runl_s[e] = (short)v[u];
-    }
-  }
+  cp_async_commit();
+  cp_async_wait0();
 }
 
-// Ring depth of the forward's operand stages: two keep three CTAs (mixed mode) on an SM, one wave of
-// tiles; the three-pass kernel (one CTA per SM, 60 KB stages) takes three, two blocks of run-record
-// copies in flight per builder thread.
+// Forward operand stages.  One pass (mixed mode): whole 64-column blocks, two stages, three CTAs an SM.
+// Three passes: blocks of 32 columns (four intervals, 64-byte rows) in stages of 30 KB: with 64-column
+// stages one CTA filled an SM, and its builders, its chain of dependent MMAs (about 125 clocks each) and
+// its epilogue took turns (12,288 water atoms 85 -> 71 us, 32,000 copper atoms 150 -> 131 us, the skipped
+// blocks included).
 template <int NPASS>
-struct MomStages {
-  static constexpr int value = NPASS == 1 ? 2 : 3;
+struct MomFwd {
+  static constexpr bool halves = NPASS == 3;
+  static constexpr int cols = halves ? 32 : 64;   // K columns of a block
+  static constexpr int a_bytes = kRows * cols * 2;  // one part of A
 };
+// The ring of S stages and the run lists; the epilogue's T tile ([32][npad + 1][4] FP32) lies over both.
+__host__ __device__ inline size_t fwd_region(int npass, int npad, int ncl, int S) {
+  const size_t ring = (size_t)S * (npass == 1 ? 1 : 2) * (kRows + npad) * (npass == 1 ? 128 : 64);
+  const size_t lists = ring + (size_t)kAtoms * ncl * 2, smt = (size_t)kAtoms * (npad + 1) * 16;
+  return ((lists > smt ? lists : smt) + 15) & ~(size_t)15;
+}
 
-
-// Largest 8-interval group holding a neighbour of each type, over the tile's atoms (the first
-// run of each list has the largest interval; runl_s holds the tile's run lists).
-__device__ __forceinline__ void tile_groups(const MomArgs& g, const short* runl_s, int a, int* ghi) {
+// The tile's schedule, by one warp (lane = atom of the tile, real or not): from the run masks, or the
+// largest group of each type (the first run of each list has the largest interval; runl_s holds the
+// tile's run lists).
+template <bool HALVES>
+__device__ __forceinline__ void build_sched(const MomArgs& g, const short* runl_s, int row, bool real, int lane,
+                                            Sched& sc, unsigned short* entries) {
+  int n = 0;
   for (int t = 0; t < g.ntypes; ++t) {
-    const int l = runl_s[a * g.nc + g.sel_off[t]];
-    if (l >= 0) atomicMax(&ghi[t], l >> 3);
+    if (g.run_mask) {
+      uint2 m = make_uint2(0u, 0u);
+      if (real) m = __ldg(g.run_mask + (long)row * g.ntypes + t);
+      m.x = __reduce_or_sync(0xffffffffu, m.x);
+      m.y = __reduce_or_sync(0xffffffffu, m.y);
+      // lane k: group 31 - k (two bits of the 64-bit mask), so that groups come out descending
+      const int grp = 31 - lane;
+      const unsigned w = (grp < 16 ? m.x >> (2 * grp) : m.y >> (2 * grp - 32)) & 3u;
+      const int cnt = HALVES ? __popc(w) : (w != 0u);
+      int incl = cnt;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += x;
+      }
+      int at = n + incl - cnt;
+      if (HALVES) {
+        if (w & 1u) entries[at++] = (unsigned short)((t << 8) | (2 * grp));
+        if (w & 2u) entries[at] = (unsigned short)((t << 8) | (2 * grp + 1));
+      } else if (w) {
+        entries[at] = (unsigned short)((t << 8) | grp);
+      }
+      n += __shfl_sync(0xffffffffu, incl, 31);
+    } else {
+      const int l = runl_s[lane * g.ncl + g.sel_off[t]];
+      const int hi = __reduce_max_sync(0xffffffffu, l >= 0 ? l >> 3 : -1);
+      if (lane == 0) sc.ghi[t] = hi;
+      n += (hi + 1) * (HALVES ? 2 : 1);
+    }
   }
+  if (lane == 0) sc.n = n;
 }
 
 // =============================================================================================
@@ -292,6 +327,7 @@ __global__ void __launch_bounds__(256, 3)
   dnext = disp_batch(task + wstride, task + wstride < ntask ? g.sel_off[(task + wstride) % pc.ntypes] : 0);
   const int i = g.disp ? -1 : g.perm[p];  // with displacements: read only for an exact pair
   const long rbase = (long)p * pc.nc + kb0;  // first run record of this list
+  short* runl = g.run_l + (long)p * g.ncl + kb0;
   // Mixed mode: the displacement in FP32 as (l_j + delta . h_c) - l_i from the cell-local
   // positions of the list build (delta: the virtual-cell offset of the image of j), with the
   // list build's error bound; pairs within that bound of r_c take the exact FP64 displacement.
@@ -310,6 +346,7 @@ __global__ void __launch_bounds__(256, 3)
   int carry_l = -1;                          // interval of the run open at the last batch's end
   int nruns = 0;
   bool oor = false;
+  unsigned mask_lo = 0, mask_hi = 0;  // bit l >> 2 of the runs so far
   for (int base = kb0; base < kb1; base += 32) {
     const int k = base + lane;
     const bool in = k < kb1;
@@ -440,7 +477,7 @@ __global__ void __launch_bounds__(256, 3)
       for (int e = 0; e < 24; ++e) v[e] += carry[e];
     if (carry_l >= 0 && !cont0 && lane == 0) {  // the open run ended exactly at the batch boundary
       const long rec = rbase + nruns - 1;
-      g.run_l[rec] = carry_l;
+      runl[nruns - 1] = (short)carry_l;
       uint4* dst = g.run_rec + rec * 4 * PARTS;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
@@ -460,7 +497,7 @@ __global__ void __launch_bounds__(256, 3)
     const int open = (!ends && lastvalid >= 0) ? 31 - __clz(segmask & (0xffffffffu >> (31 - lastvalid))) : -1;
     if (seg && lane != open) {
       const long rec = rbase + myrun;
-      g.run_l[rec] = lk;
+      runl[myrun] = (short)lk;
       uint4* dst = g.run_rec + rec * 4 * PARTS;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
@@ -480,36 +517,44 @@ __global__ void __launch_bounds__(256, 3)
     }
     __syncwarp();
     nruns += __popc(headmask);
+    if (g.run_mask) {
+      const int b = lk >> 2;
+      mask_lo |= __reduce_or_sync(0xffffffffu, valid && b < 32 ? 1u << b : 0u);
+      mask_hi |= __reduce_or_sync(0xffffffffu, valid && b >= 32 ? 1u << (b - 32) : 0u);
+    }
     if (ends) break;  // warp-uniform: the rest of the block is padding
   }
-  if (lane == 0 && nruns < kb1 - kb0) g.run_l[rbase + nruns] = -1;
+  if (lane == 0 && nruns < kb1 - kb0) runl[nruns] = -1;
+  if (lane == 0 && g.run_mask) g.run_mask[task] = make_uint2(mask_lo, mask_hi);
   if (__any_sync(0xffffffffu, oor) && lane == 0) atomicOr(g.table_range, 1);
   }
 }
 
 // =============================================================================================
 // Forward: T and D.  Thread r < 128 owns A row r = (atom r / 4, component r % 4): for every
-// 8-interval block it copies the chunks of its atom's runs in the block from the run records
+// scheduled block it copies the chunks of its atom's runs in the block from the run records
 // (cp.async, already in operand format) and clears the chunks of empty intervals; the copies of
 // block kb are released to the MMA once they have landed, up to S - 1 blocks later.
 // =============================================================================================
-template <int NPASS, int NPAD>
-__global__ void __launch_bounds__(kMomThreads, NPASS == 1 ? 3 : 1)
+template <int NPASS, int NPAD, int S>
+__global__ void __launch_bounds__(kMomThreads, NPASS == 1 ? 3 : 2)
     k_mom_fwd(const __grid_constant__ CUtensorMap bhi, const __grid_constant__ CUtensorMap blo, const MomArgs g) {
   constexpr int PARTS = NPASS == 1 ? 1 : 2;
-  constexpr int S = MomStages<NPASS>::value;
+  constexpr bool HALVES = MomFwd<NPASS>::halves;
+  constexpr int IV = MomFwd<NPASS>::cols / 8;  // intervals of a block
   constexpr int D = S - 1;  // blocks in flight per builder thread
-  constexpr int B_BYTES = NPAD * 128;
-  constexpr int STAGE = PARTS * (kABlock + B_BYTES);
+  constexpr int A_BYTES = MomFwd<NPASS>::a_bytes;
+  constexpr int B_BYTES = NPAD * MomFwd<NPASS>::cols * 2;
+  constexpr int STAGE = PARTS * (A_BYTES + B_BYTES);
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  short* runl_s = reinterpret_cast<short*>(smem + S * STAGE);  // [32 atoms][nc] run intervals of the tile
-  uint64_t* full = reinterpret_cast<uint64_t*>(runl_s + kAtoms * g.nc);
+  short* runl_s = reinterpret_cast<short*>(smem + S * STAGE);  // [32 atoms][ncl] run intervals of the tile
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + fwd_region(NPASS, NPAD, g.ncl, S));
   uint64_t* empty = full + S;
   uint64_t* accf = empty + S;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(accf + 1);
-  int* ghi = reinterpret_cast<int*>(tmem_holder + 1);
+  __shared__ Sched sc;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int ti = 0;
@@ -523,7 +568,6 @@ __global__ void __launch_bounds__(kMomThreads, NPASS == 1 ? 3 : 1)
       mbar_init(&empty[s], 1);
     }
     mbar_init(accf, 1);
-    for (int t = 0; t < DP_MAX_TYPES; ++t) ghi[t] = -1;
     mbar_fence_init();
   }
   if (warp == 4) tmem_alloc(tmem_holder, 128);
@@ -532,15 +576,20 @@ __global__ void __launch_bounds__(kMomThreads, NPASS == 1 ? 3 : 1)
   const int r = threadIdx.x;
   const int ae = r >> 2, c = r & 3;
   const int pe = row0 + ae;
+  const bool masks = g.run_mask != nullptr;
+  unsigned short* entries = masks ? reinterpret_cast<unsigned short*>(tmem_holder + 1) : nullptr;
+  if (warp == 5 && masks) build_sched<HALVES>(g, nullptr, row0 + lane, row0 + lane < row_end, lane, sc, entries);
   stage_runs(g, row0, row_end, runl_s, threadIdx.x, kMomThreads);
   __syncthreads();
-  if (warp == 0) tile_groups(g, runl_s, lane, ghi);
+  if (!masks) {
+    if (warp == 0) build_sched<HALVES>(g, runl_s, row0 + lane, row0 + lane < row_end, lane, sc, entries);
+    __syncthreads();
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_holder;
-  int nkb = 0;
-  for (int t = 0; t < g.ntypes; ++t) nkb += ghi[t] + 1;
+  const int nkb = sc.n;
 
   if (warp == 5) {
     if (lane == 0) {
@@ -549,11 +598,11 @@ __global__ void __launch_bounds__(kMomThreads, NPASS == 1 ? 3 : 1)
       for (int kb = 0; kb < nkb; ++kb) {
         const int s = kb % S;
         if (kb >= S && !mbar_wait(&empty[s], ((kb / S) - 1) & 1, g.err)) break;
-        int t, grp;
-        block_of(kb, ghi, g.ntypes, t, grp);
-        unsigned char* bs = smem + s * STAGE + PARTS * kABlock;
+        int t, grp, h;
+        block_of<HALVES>(sc, entries, kb, g.ntypes, t, grp, h);
+        unsigned char* bs = smem + s * STAGE + PARTS * A_BYTES;
         mbar_expect_tx(&full[s], PARTS * B_BYTES);
-        const int x = (t * g.lcp + 8 * grp) * 8;
+        const int x = (t * g.lcp + 8 * grp + IV * h) * 8;
         tma_load_2d(bs, &bhi, &full[s], x, ti * NPAD);
         if (PARTS == 2) tma_load_2d(bs + B_BYTES, &blo, &full[s], x, ti * NPAD);
         issued = kb + 1;
@@ -575,10 +624,11 @@ __global__ void __launch_bounds__(kMomThreads, NPASS == 1 ? 3 : 1)
         }
         tc_fence_after();
         const uint32_t sa = su32(smem + s * STAGE);
-        const uint64_t ah = sdesc_sw128(sa), al = sdesc_sw128(sa + kABlock);
-        const uint64_t bh = sdesc_sw128(sa + PARTS * kABlock), bl = sdesc_sw128(sa + PARTS * kABlock + B_BYTES);
+        auto desc = [](uint32_t a) { return HALVES ? sdesc_sw64(a) : sdesc_sw128(a); };
+        const uint64_t ah = desc(sa), al = desc(sa + A_BYTES);
+        const uint64_t bh = desc(sa + PARTS * A_BYTES), bl = desc(sa + PARTS * A_BYTES + B_BYTES);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < MomFwd<NPASS>::cols / 16; ++k) {
           mma_f16(tmem, ah + 2 * k, bh + 2 * k, idesc, (kb | k) != 0);
           if (NPASS == 3) {
             mma_f16(tmem, ah + 2 * k, bl + 2 * k, idesc, 1);
@@ -595,13 +645,15 @@ __global__ void __launch_bounds__(kMomThreads, NPASS == 1 ? 3 : 1)
     }
   } else {
     // ---- operand builders ----
-    int cur_t = -1, ptr = 0, selt = 0;
+    int cur_t = -1, cur_g = -1, selt = 0;
+    int pbeg = 0, pmid = 0, pend = 0;  // the group's runs: [pbeg, pmid) upper half, [pmid, pend) lower half
     long rbase = 0;
     bool dead = false;  // after a timed-out wait: stop waiting, keep going through the blocks
-    const uint32_t rowoff0 = (uint32_t)((r >> 3) * 1024 + (r & 7) * 128);
+    const uint32_t rowoff0 = HALVES ? (uint32_t)(r * 64) : (uint32_t)((r >> 3) * 1024 + (r & 7) * 128);
+    const int xr = HALVES ? (r >> 1) & 3 : r & 7;  // swizzle of the row's 16-byte chunks
     for (int kb = 0; kb < nkb; ++kb) {
-      int t, grp;
-      block_of(kb, ghi, g.ntypes, t, grp);
+      int t, grp, h;
+      block_of<HALVES>(sc, entries, kb, g.ntypes, t, grp, h);
       const int s = kb % S;
       if (kb >= D) {  // block kb - D: its copies have landed (the D - 1 later groups may still be in flight)
         cp_async_wait<D - 1>();
@@ -611,29 +663,34 @@ __global__ void __launch_bounds__(kMomThreads, NPASS == 1 ? 3 : 1)
       if (kb >= S && !dead && !mbar_wait(&empty[s], ((kb / S) - 1) & 1, g.err)) dead = true;
       if (t != cur_t) {
         cur_t = t;
+        cur_g = -1;
         selt = g.sel_off[t + 1] - g.sel_off[t];
-        ptr = 0;
+        pend = 0;
         rbase = (long)pe * g.nc + g.sel_off[t];
       }
-      const short* myruns = runl_s + ae * g.nc + g.sel_off[t];
+      const short* myruns = runl_s + ae * g.ncl + g.sel_off[t];
+      if (grp != cur_g) {  // runs descend along the list, and end with -1
+        cur_g = grp;
+        pbeg = pend;
+        while (HALVES && pend < selt && myruns[pend] >= 8 * grp + IV) ++pend;
+        pmid = HALVES ? pend : pbeg;
+        while (pend < selt && myruns[pend] >= 8 * grp) ++pend;
+      }
       unsigned char* ahi = smem + s * STAGE;
-      unsigned char* alo = ahi + kABlock;
+      unsigned char* alo = ahi + A_BYTES;
       unsigned covered = 0;
-      while (ptr < selt) {
-        const int l = myruns[ptr];
-        if (l < 8 * grp) break;  // also the end marker -1
-        const int q = (l - 8 * grp) & 7;
-        const uint32_t off = rowoff0 + (uint32_t)((q ^ (r & 7)) << 4);
-        const uint4* src = g.run_rec + ((rbase + ptr) * 4 + c) * PARTS;
+      for (int p = HALVES && h ? pbeg : pmid, e = HALVES && h ? pmid : pend; p < e; ++p) {
+        const int q = (myruns[p] - 8 * grp - IV * h) & (IV - 1);
+        const uint32_t off = rowoff0 + (uint32_t)((q ^ xr) << 4);
+        const uint4* src = g.run_rec + ((rbase + p) * 4 + c) * PARTS;
         cp_async16(ahi + off, src);
         if (PARTS == 2) cp_async16(alo + off, src + 1);
         covered |= 1u << q;
-        ++ptr;
       }
 #pragma unroll
-      for (int q = 0; q < 8; ++q)
+      for (int q = 0; q < IV; ++q)
         if (!((covered >> q) & 1u)) {
-          const uint32_t off = rowoff0 + (uint32_t)((q ^ (r & 7)) << 4);
+          const uint32_t off = rowoff0 + (uint32_t)((q ^ xr) << 4);
           *reinterpret_cast<uint4*>(ahi + off) = make_uint4(0u, 0u, 0u, 0u);
           if (PARTS == 2) *reinterpret_cast<uint4*>(alo + off) = make_uint4(0u, 0u, 0u, 0u);
         }
@@ -895,11 +952,10 @@ __global__ void __launch_bounds__(kRows)
 // run of its atom in the block, the six values of its interval (scaled back by 2^ex / Nc) to the
 // run's P record; the per-slot part of the backward is k_force_mom.
 // =============================================================================================
-template <int NPASS, int NPAD>
+template <int NPASS, int NPAD, int S>
 __global__ void __launch_bounds__(kMomThreads, 1)
     k_mom_bwd(const __grid_constant__ CUtensorMap bhi, const __grid_constant__ CUtensorMap blo, const MomArgs g) {
   constexpr int PARTS = NPASS == 1 ? 1 : 2;
-  constexpr int S = BwdDepth<NPASS>::stages;
   constexpr int kAccBufs = BwdDepth<NPASS>::acc;
   constexpr int A_BYTES = 2 * kABlock;  // K = m in two 64-column blocks
   constexpr int B_KBLK = 64 * 128;      // 64 rows (8 intervals x 8 powers) x 128 B
@@ -910,8 +966,8 @@ __global__ void __launch_bounds__(kMomThreads, 1)
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   unsigned char* As = smem;                      // PARTS x A_BYTES, dE/dT rows (A operand)
   unsigned char* ring = smem + PARTS * A_BYTES;  // B stages
-  short* runl_s = reinterpret_cast<short*>(ring + S * B_STAGE);  // [32 atoms][nc] run intervals of the tile
-  int* ex_s = reinterpret_cast<int*>(runl_s + kAtoms * g.nc);       // [128] power-of-two scale of each row
+  short* runl_s = reinterpret_cast<short*>(ring + S * B_STAGE);  // [32 atoms][ncl] run intervals of the tile
+  int* ex_s = reinterpret_cast<int*>(runl_s + kAtoms * g.ncl);       // [128] power-of-two scale of each row
   uint64_t* bar = reinterpret_cast<uint64_t*>(ex_s + kRows);
   uint64_t* bfull = bar;
   uint64_t* bempty = bar + S;
@@ -919,7 +975,7 @@ __global__ void __launch_bounds__(kMomThreads, 1)
   uint64_t* accfull = afull + 1;     // [kAccBufs]
   uint64_t* accempty = accfull + kAccBufs;  // [kAccBufs]
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(accempty + kAccBufs);
-  int* ghi = reinterpret_cast<int*>(tmem_holder + 1);
+  __shared__ Sched sc;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int ti = 0;
@@ -937,7 +993,6 @@ __global__ void __launch_bounds__(kMomThreads, 1)
       mbar_init(&accfull[b], 1);
       mbar_init(&accempty[b], kRows);
     }
-    for (int t = 0; t < DP_MAX_TYPES; ++t) ghi[t] = -1;
     mbar_fence_init();
   }
   if (warp == 4) tmem_alloc(tmem_holder, 64 * kAccBufs);
@@ -946,15 +1001,20 @@ __global__ void __launch_bounds__(kMomThreads, 1)
   const int r = threadIdx.x;
   const int ae = r >> 2, c = r & 3;
   const int pe = row0 + ae;
+  const bool masks = g.run_mask != nullptr;
+  unsigned short* entries = masks ? reinterpret_cast<unsigned short*>(tmem_holder + 1) : nullptr;
+  if (warp == 5 && masks) build_sched<false>(g, nullptr, row0 + lane, row0 + lane < row_end, lane, sc, entries);
   stage_runs(g, row0, row_end, runl_s, threadIdx.x, kMomThreads);
   __syncthreads();
-  if (warp == 0) tile_groups(g, runl_s, lane, ghi);
+  if (!masks) {
+    if (warp == 0) build_sched<false>(g, runl_s, row0 + lane, row0 + lane < row_end, lane, sc, entries);
+    __syncthreads();
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_holder;
-  int nch = 0;
-  for (int t = 0; t < g.ntypes; ++t) nch += ghi[t] + 1;
+  const int nch = sc.n;
 
   if (warp == 5) {
     if (lane == 0) {
@@ -963,8 +1023,8 @@ __global__ void __launch_bounds__(kMomThreads, 1)
       for (int ch = 0; ch < nch; ++ch) {
         const int s = ch % S;
         if (ch >= S && !mbar_wait(&bempty[s], ((ch / S) - 1) & 1, g.err)) break;
-        int t, grp;
-        block_of(ch, ghi, g.ntypes, t, grp);
+        int t, grp, h;
+        block_of<false>(sc, entries, ch, g.ntypes, t, grp, h);
         unsigned char* bs = ring + s * B_STAGE;
         mbar_expect_tx(&bfull[s], B_STAGE);
         const int y = ((ti * g.ntypes + t) * g.lcp + 8 * grp) * 8;
@@ -990,34 +1050,50 @@ __global__ void __launch_bounds__(kMomThreads, 1)
       bool ok = mbar_wait(afull, 0, g.err);
       // ---- MMA issuer ----
       const uint32_t idesc = idesc_f16(kRows, 64, NPASS == 1 ? 0 : 1);
-      for (int ch = 0; ok && ch < nch; ++ch) {
-        const int s = ch % S, buf = ch % kAccBufs;
-        if (!mbar_wait(&bfull[s], (ch / S) & 1, g.err)) {
-          ok = false;
-          break;
+      // Four stages: two chunks at a time, their MMAs interleaved.  Each accumulator's MMAs are a chain
+      // of about 125 clocks a link; two chains fill the gaps of one.  With three the loads of the next
+      // pair would wait (32,000 atoms of 500 neighbours: 125 us one at a time, 142 us in pairs).
+      constexpr int PAIR = S >= 4 ? 2 : 1;
+      for (int ch0 = 0; ok && ch0 < nch; ch0 += PAIR) {
+        const int np = min(PAIR, nch - ch0);
+        for (int j = 0; ok && j < np; ++j) {
+          const int ch = ch0 + j, s = ch % S, buf = ch % kAccBufs;
+          ok = mbar_wait(&bfull[s], (ch / S) & 1, g.err);
+          if (ok && ch >= kAccBufs) ok = mbar_wait(&accempty[buf], ((ch / kAccBufs) - 1) & 1, g.err);
         }
-        if (ch >= kAccBufs && !mbar_wait(&accempty[buf], ((ch / kAccBufs) - 1) & 1, g.err)) {
-          ok = false;
-          break;
-        }
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t sa = su32(As), sb = su32(ring + s * B_STAGE);
-        const uint32_t acc = tmem + (uint32_t)(buf * 64);
+        const uint32_t sa = su32(As);
 #pragma unroll
         for (int ks = 0; ks < KSTEPS; ++ks) {
           const uint32_t kbk = (uint32_t)(ks >> 2), ko = (uint32_t)(ks & 3) * 2;
           const uint64_t ah = sdesc_sw128(sa + kbk * kABlock) + ko;
-          const uint64_t bh = sdesc_sw128(sb + kbk * B_KBLK) + ko;
-          mma_f16(acc, ah, bh, idesc, ks != 0);
+          const uint64_t al = sdesc_sw128(sa + A_BYTES + kbk * kABlock) + ko;
+          auto operands = [&](int j, uint32_t& acc, uint64_t& bh, uint64_t& bl) {
+            const int ch = ch0 + j;
+            const uint32_t sb = su32(ring + (ch % S) * B_STAGE);
+            acc = tmem + (uint32_t)((ch % kAccBufs) * 64);
+            bh = sdesc_sw128(sb + kbk * B_KBLK) + ko;
+            bl = sdesc_sw128(sb + 2 * B_KBLK + kbk * B_KBLK) + ko;
+          };
+          uint32_t acc0, acc1;
+          uint64_t bh0, bl0, bh1, bl1;
+          operands(0, acc0, bh0, bl0);
+          operands(PAIR - 1, acc1, bh1, bl1);
+          const bool two = np == 2;
+          mma_f16(acc0, ah, bh0, idesc, ks != 0);
+          if (two) mma_f16(acc1, ah, bh1, idesc, ks != 0);
           if (NPASS == 3) {
-            const uint64_t al = sdesc_sw128(sa + A_BYTES + kbk * kABlock) + ko;
-            const uint64_t bl = sdesc_sw128(sb + 2 * B_KBLK + kbk * B_KBLK) + ko;
-            mma_f16(acc, ah, bl, idesc, 1);
-            mma_f16(acc, al, bh, idesc, 1);
+            mma_f16(acc0, ah, bl0, idesc, 1);
+            if (two) mma_f16(acc1, ah, bl1, idesc, 1);
+            mma_f16(acc0, al, bh0, idesc, 1);
+            if (two) mma_f16(acc1, al, bh1, idesc, 1);
           }
         }
-        mma_commit(&bempty[s]);
-        mma_commit(&accfull[buf]);
+        for (int j = 0; j < np; ++j) {
+          mma_commit(&bempty[(ch0 + j) % S]);
+          mma_commit(&accfull[(ch0 + j) % kAccBufs]);
+        }
       }
       if (ok && nch > 0) atomicAdd(&g.mma_blocks[1], (unsigned)nch);
     }
@@ -1071,15 +1147,15 @@ __global__ void __launch_bounds__(kMomThreads, 1)
       }
       tc_fence_before();
       mbar_arrive(&accempty[buf]);
-      int t, grp;
-      block_of(ch, ghi, g.ntypes, t, grp);
+      int t, grp, h;
+      block_of<false>(sc, entries, ch, g.ntypes, t, grp, h);
       if (t != cur_t) {
         cur_t = t;
         selt = g.sel_off[t + 1] - g.sel_off[t];
         ptr = 0;
         rbase = (long)pe * g.nc + g.sel_off[t];
       }
-      const short* myruns = runl_s + ae * g.nc + g.sel_off[t];
+      const short* myruns = runl_s + ae * g.ncl + g.sel_off[t];
       while (ptr < selt) {
         const int l = myruns[ptr];
         if (l < 8 * grp) break;  // also the end marker -1
@@ -1265,17 +1341,15 @@ __global__ void k_mom_tables(const double* __restrict__ tab, int ntypes, int one
   }
 }
 
-size_t fwd_smem(int npass, int npad, int nc) {
-  const int parts = npass == 1 ? 1 : 2, S = npass == 1 ? MomStages<1>::value : MomStages<3>::value;
-  return (size_t)S * parts * (kABlock + npad * 128) + (size_t)kAtoms * nc * 2 + (2 * S + 1) * 8 + 4 +
-         4 * DP_MAX_TYPES + 1024 + 64;
+size_t sched_smem(const MomArgs& g) { return g.run_mask ? kSchedMax * sizeof(unsigned short) : 0; }
+size_t fwd_smem(const MomArgs& g, int npass, int npad, int S) {
+  return fwd_region(npass, npad, g.ncl, S) + (2 * S + 1) * 8 + 16 + 1024 + sched_smem(g);
 }
-size_t bwd_smem(int npass, int nc) {
+size_t bwd_smem(const MomArgs& g, int npass, int S) {
   const int parts = npass == 1 ? 1 : 2;
-  const int S = npass == 1 ? BwdDepth<1>::stages : BwdDepth<3>::stages;
   const int nacc = npass == 1 ? BwdDepth<1>::acc : BwdDepth<3>::acc;
-  return (size_t)parts * 2 * kABlock + S * (size_t)parts * 2 * 64 * 128 + (size_t)kAtoms * nc * 2 +
-         kRows * 4 + (2 * S + 1 + 2 * nacc) * 8 + 4 + 4 * DP_MAX_TYPES + 1024 + 64;
+  return (size_t)parts * 2 * kABlock + S * (size_t)parts * 2 * 64 * 128 + (size_t)kAtoms * g.ncl * 2 +
+         kRows * 4 + (2 * S + 1 + 2 * nacc) * 8 + 16 + 1024 + sched_smem(g);
 }
 
 template <int NPASS, int NPAD>
@@ -1284,13 +1358,38 @@ int launch_mom(const DeviceModel& m, const MomArgs& g, int tiles, int which, boo
   if (which == 1) {
     DP_CUDA_TRY(launch_chain(pdl, k_mom_gT<NPASS, NPAD>, dim3(tiles, kAtoms / kGroupAtoms), dim3(kRows), 0, st, g));
   } else if (which == 0) {
-    const size_t sm = fwd_smem(NPASS, NPAD, g.nc);
-    DP_CUDA_TRY(allow_max_smem(k_mom_fwd<NPASS, NPAD>));
-    DP_CUDA_TRY(launch_chain(pdl, k_mom_fwd<NPASS, NPAD>, dim3(tiles), dim3(kMomThreads), sm, st, maps[0], maps[1], g));
+    // Three passes: with more tiles than SMs three stages where two such CTAs share an SM, else two; with
+    // fewer there is nobody to share with, and six keep twice the copies in flight.
+    constexpr size_t kHalfSm = 113 * 1024, kWholeSm = 226 * 1024;
+    auto kernel = k_mom_fwd<NPASS, NPAD, 2>;
+    int S = 2;
+    if constexpr (NPASS == 3) {
+      if (tiles <= sm_count() && fwd_smem(g, NPASS, NPAD, 6) <= kWholeSm) {
+        S = 6;
+        kernel = k_mom_fwd<NPASS, NPAD, 6>;
+      } else if (fwd_smem(g, NPASS, NPAD, 3) <= kHalfSm) {
+        S = 3;
+        kernel = k_mom_fwd<NPASS, NPAD, 3>;
+      }
+    }
+    DP_CUDA_TRY(allow_max_smem(kernel));
+    DP_CUDA_TRY(launch_chain(pdl, kernel, dim3(tiles), dim3(kMomThreads), fwd_smem(g, NPASS, NPAD, S), st, maps[0],
+                             maps[1], g));
   } else {
-    const size_t sm = bwd_smem(NPASS, g.nc);
-    DP_CUDA_TRY(allow_max_smem(k_mom_bwd<NPASS, NPAD>));
-    DP_CUDA_TRY(launch_chain(pdl, k_mom_bwd<NPASS, NPAD>, dim3(tiles), dim3(kMomThreads), sm, st, maps[2], maps[3], g));
+    auto kernel = k_mom_bwd<NPASS, NPAD, NPASS == 3 ? 3 : 2>;
+    int S = NPASS == 3 ? 3 : 2;
+    if constexpr (NPASS == 3) {
+      if (bwd_smem(g, NPASS, 4) <= 226 * 1024) {
+        S = 4;
+        kernel = k_mom_bwd<NPASS, NPAD, 4>;
+      } else if (bwd_smem(g, NPASS, 3) > 226 * 1024) {  // lists of more than 1,000 slots
+        S = 2;
+        kernel = k_mom_bwd<NPASS, NPAD, 2>;
+      }
+    }
+    const size_t sm = bwd_smem(g, NPASS, S);
+    DP_CUDA_TRY(allow_max_smem(kernel));
+    DP_CUDA_TRY(launch_chain(pdl, kernel, dim3(tiles), dim3(kMomThreads), sm, st, maps[2], maps[3], g));
   }
   DP_CUDA_TRY(cudaGetLastError());
   return DP_OK;
@@ -1350,8 +1449,9 @@ int build_mom_tables(DeviceModel& m) {
   DP_CUDA_TRY(cudaDeviceSynchronize());
   m.mom_maps.assign(4 * sizeof(CUtensorMap), 0);
   CUtensorMap* maps = reinterpret_cast<CUtensorMap*>(m.mom_maps.data());
-  int rc = make_tmap_bf16(&maps[0], fwd_hi, (long)nt * npad, kcols, npad);
-  if (rc == DP_OK) rc = make_tmap_bf16(&maps[1], parts == 2 ? fwd_lo : fwd_hi, (long)nt * npad, kcols, npad);
+  const int fwd_cols = npass == 1 ? MomFwd<1>::cols : MomFwd<3>::cols;
+  int rc = make_tmap_bf16(&maps[0], fwd_hi, (long)nt * npad, kcols, npad, fwd_cols);
+  if (rc == DP_OK) rc = make_tmap_bf16(&maps[1], parts == 2 ? fwd_lo : fwd_hi, (long)nt * npad, kcols, npad, fwd_cols);
   if (rc == DP_OK) rc = make_tmap_bf16(&maps[2], bwd_hi, (long)nt * nt * lcp * 8, 128, 64);
   if (rc == DP_OK) rc = make_tmap_bf16(&maps[3], parts == 2 ? bwd_lo : bwd_hi, (long)nt * nt * lcp * 8, 128, 64);
   if (rc != DP_OK) return rc;
@@ -1376,7 +1476,10 @@ int run_mom(const DeviceModel& m, const PathConst& pc, const PathIO& io, Arena& 
   float4* envU = ar.get<float4>(slots);
   float4* envB = ar.get<float4>(slots);
   int* slot_run = ar.get<int>(slots);
-  int* run_l = ar.get<int>(slots);
+  const int ncl = (pc.nc + 7) & ~7;
+  short* run_l = ar.get<short>(N * ncl);
+  // (lists of more slots than the search keeps per type leave no room for the schedule's entries)
+  uint2* run_mask = m.mom_lcp <= 256 && pc.nc <= 1024 ? ar.get<uint2>(N * pc.ntypes) : nullptr;
   // run moments (forward) and run P (backward) share one buffer: the moments are dead by then
   void* runs = ar.get<float4>(slots * 8 > slots * 4 * parts ? slots * 8 : slots * 4 * parts);
   const long max_tiles = (N + kAtoms - 1) / kAtoms + pc.ntypes;  // every type's last tile may be short
@@ -1432,6 +1535,8 @@ int run_mom(const DeviceModel& m, const PathConst& pc, const PathIO& io, Arena& 
   g.envB = envB;
   g.slot_run = slot_run;
   g.run_l = run_l;
+  g.ncl = ncl;
+  g.run_mask = run_mask;
   g.run_rec = reinterpret_cast<uint4*>(runs);
   g.run_P = reinterpret_cast<float4*>(runs);
   g.p_bf16 = bf16 ? 1 : 0;

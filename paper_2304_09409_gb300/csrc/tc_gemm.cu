@@ -35,7 +35,7 @@ using namespace ptx;
 // epilogues) share an SM.  Split operands (NP = 3) carry high and low parts of both tiles per
 // stage (48 KB at BN = 64): two stages, so that two CTAs share an SM and one's epilogue runs
 // while the other's operands stream in -- unless the grid does not fill the SMs, when nothing is to
-// share one and four stages keep the loads ahead (K = 1,600: 24 -> 15 us).
+// share one and four stages keep the loads ahead (K = 1,600: 24.2 -> 22.8 us; the chain of dependent MMAs is the rest).
 __host__ __device__ inline uint32_t stage_bytes_of(int BN, int NP) {
   return (uint32_t)(NP == 3 ? 2 : 1) * (uint32_t)(BM * BK * 2 + BN * BK * 2);
 }
