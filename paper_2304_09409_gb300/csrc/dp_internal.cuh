@@ -253,6 +253,9 @@ struct NlExtras {
   // padding beyond that batch may stay unwritten
   bool lean;
   bool counts_clear;  // cell_count is zero already
+  // optional: positions [natoms][2] and image translations [nframes][27][2] as two-float pairs,
+  // {high x, y, z, largest |high|}, {low x, y, z, 0}
+  float4 *pos2, *tshift2;
 };
 // Cell arrays are indexed by (type, cell): cell_count [ntypes * ncells_total], cell_start
 // [ntypes * ncells_total + 1]; per atom its key and rank within the key (atom_key, int2), its

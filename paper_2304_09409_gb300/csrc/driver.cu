@@ -227,6 +227,7 @@ struct Bufs {
   unsigned char* ftab;
   int* atom_frame;
   double* tshift;
+  float4 *pos2, *tshift2;  // three-pass moment path: positions and image translations as two floats
   int *perm, *type_start;
   double *energy, *virial, *force, *atom_energy, *atom_virial, *cpart, *epart;
   int* fcount;  // finished chunks per frame (k_chunk_sums)
@@ -255,6 +256,10 @@ void carve(Arena& ar, const DeviceModel& m, const FrameTables& T, bool own_nlist
   b.ftab = ar.get<unsigned char>((long)T.bytes);
   if (T.F > 1) b.atom_frame = ar.get<int>(N);
   b.tshift = ar.get<double>(81L * T.F);
+  if (own_nlist && m.compressed && m.mom_npass == 3) {
+    b.pos2 = ar.get<float4>(2 * N);
+    b.tshift2 = ar.get<float4>(54L * T.F);
+  }
   b.perm = ar.get<int>(N);
   b.type_start = ar.get<int>(DP_MAX_TYPES + 1);
   if (host_e) b.energy = ar.get<double>(T.F);
@@ -467,7 +472,7 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
       // the moment path reads its list in batches
       const bool lean = m.compressed && m.cfg.descriptor == DP_DESC_SE_E2_A && m.mom_npass != 0;
       NlExtras ex{b.perm, b.type_start, chk, d_boxes, T.periodic ? F : 0, T.periodic ? b.tshift : nullptr, b.disp,
-                  false, lean, true};
+                  false, lean, true, b.pos2, b.tshift2};
       ProfScope _ps(&md->prof, "nlist", s, nlist_launches(L, m.cfg.ntypes));
       const NlScratch sc{b.cell_count, b.cell_start, b.atom_key, b.atom_l, b.atom_m, b.sorted_l, b.sorted_m};
       DP_CUDA_TRY(launch_nlist_build(L, m.cfg.ntypes, dcoord, dtype, sc, b.nl_j, b.nl_code, b.counts, md->status, s,
@@ -508,6 +513,8 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
     io.atom_virial = b.atom_virial;
     io.status = md->status;
     io.epart = b.epart;
+    io.pos2 = b.pos2;
+    io.tshift2 = T.periodic ? b.tshift2 : nullptr;
     io.atom_l = own_nlist ? b.atom_l : nullptr;
     io.atom_m = own_nlist ? b.atom_m : nullptr;
     io.geoms = own_nlist ? d_geoms : nullptr;

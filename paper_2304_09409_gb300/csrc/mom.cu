@@ -75,11 +75,13 @@ struct MomArgs {
   const int* perm;
   const int* nl_j;
   // per-slot records, rows in sorted atom order [N * nc]: (s, u), (ds/dr, r, tau, l), run index
-  float4* envU;
-  float4* envB;
-  int* slot_run;
+  // per real slot: the displacement and its run << 16 | interval.  The backward evaluates the switch
+  // and tau again from them: 16 bytes a pair each way instead of 36 (32,000 atoms of 340 neighbours: 220 MB less
+  // written and read again)
+  float4* slot;
   // per-run records, run r of type block t of atom p at row p * nc + sel_off[t] + r
   short* run_l;    // [N][ncl] interval of the run (far below 2^15); -1 after the last run
+  const float4 *pos2, *tshift2;  // positions and image translations as two floats, or null
   int ncl;         // nc rounded up to 8: rows of run_l are 16-byte aligned
   uint2* run_mask; // [N][ntypes] bit l >> 2 of every run's interval, or null
   uint4* run_rec;  // moments as A-operand chunks [row][4 components][parts]
@@ -281,6 +283,48 @@ __device__ __forceinline__ void build_sched(const MomArgs& g, const short* runl_
   if (lane == 0) sc.n = n;
 }
 
+// The FP32 rounding of the exact FP64 displacement (listed_disp) from two-float positions, FP32 arithmetic
+// alone: three FP64 subtractions and conversions a pair kept the FP64 pipe, two operations a clock and SM,
+// busy for most of the kernel.  With M the largest of |x_j| + |t|, |x_i|, the two-float sum s + c below is
+// within 0.66 * 2^-43 M of the exact displacement (splits 3 * 2^-48, sums of the low parts 2^-47 + 2^-46 +
+// 2^-45.6 + 2^-45.2) and the FP64 value within 3 * 2^-53 M; the two bounds c -+ 2^-43 M round by at most
+// 0.22 * 2^-43 M.  So where both bounds give the same float, the FP64 value rounds to it too; elsewhere (about one
+// pair in a thousand) the caller takes the FP64 one.
+__device__ __forceinline__ bool two_float_disp(const MomArgs& g, const float4& hi, const float4& lo, int j, int code,
+                                               int fr, float& x0, float& x1, float& x2) {
+  float4 h = g.pos2[2L * j], l = g.pos2[2L * j + 1];
+  float m = h.w;
+  if (code != pack_shift(0, 0, 0)) {
+    int n0, n1, n2;
+    unpack_shift(code, n0, n1, n2);
+    if (!g.tshift2 || n0 < -1 || n0 > 1 || n1 < -1 || n1 > 1 || n2 < -1 || n2 > 1) return false;
+    const float4* t = g.tshift2 + 2 * (27L * fr + (n0 + 1) * 9 + (n1 + 1) * 3 + (n2 + 1));
+    const float4 th = t[0], tl = t[1];
+    m += th.w;
+    auto add = [](float& a, float& al, float b, float bl) {
+      const float s = a + b, bb = s - a, e = (a - (s - bb)) + (b - bb);
+      a = s;
+      al = (al + bl) + e;
+    };
+    add(h.x, l.x, th.x, tl.x);
+    add(h.y, l.y, th.y, tl.y);
+    add(h.z, l.z, th.z, tl.z);
+  }
+  const float tol = fmaxf(m, hi.w) * 0x1p-43f;
+  bool same = true;
+  auto sub = [&](float a, float al, float b, float bl) {
+    const float s = a - b, bb = s - a, e = (a - (s - bb)) - (b + bb);
+    const float c = (al - bl) + e;
+    const float x = s + (c - tol);
+    same = same && x == s + (c + tol);
+    return x;
+  };
+  x0 = sub(h.x, l.x, hi.x, lo.x);
+  x1 = sub(h.y, l.y, hi.y, lo.y);
+  x2 = sub(h.z, l.z, hi.z, lo.z);
+  return same;
+}
+
 // =============================================================================================
 // Per-slot records and per-run moments.  One warp takes one (atom, neighbour type) list, 32
 // slots at a time: exact FP64 displacement, FP32 switch (Eq. (switch)), interval and tau; the
@@ -291,7 +335,7 @@ __device__ __forceinline__ void build_sched(const MomArgs& g, const short* runl_
 // carried to the next).  Each run's moments are written in the backward's A-operand chunk
 // format (FP16, or BF16 high and low parts): the forward kernel copies them into its tiles
 // without conversion.  Outputs, for slot k of atom p (row p * Nc + k):
-//   envU (s, u), envB (ds/dr, r, tau, l) with l = -1 marking padding, slot_run (run index);
+//   slot (displacement, run index and interval), for real neighbours only;
 // and for run r of type block t (row p * Nc + sel_off[t] + r): run_l (-1 after the last run)
 // and run_rec.
 // =============================================================================================
@@ -337,6 +381,11 @@ __global__ void __launch_bounds__(256, 3)
   float4 li = make_float4(0.f, 0.f, 0.f, 0.f);
   int4 mi = make_int4(0, 0, 0, 0);
   const NlGeom* G = nullptr;
+  float4 l2 = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (NPASS == 3 && g.pos2) {
+    li = g.pos2[2L * i];
+    l2 = g.pos2[2L * i + 1];
+  }
   if (f32d) {
     li = g.atom_l[i];
     mi = g.atom_m[i];
@@ -358,11 +407,11 @@ __global__ void __launch_bounds__(256, 3)
     const bool valid = g.disp ? dd.w >= 0.f : j >= 0;
     int l = INT_MAX;
     float r = 0.f, s = 0.f, ds = 0.f, u[3] = {0.f, 0.f, 0.f}, tau = 0.f;
+    float x0 = 0.f, x1 = 0.f, x2 = 0.f;
     if (valid) {
       // the FP32 displacement: handed over by the list build, or formed from the gathered
       // cell-local positions, or (near r_c) rounded from the exact FP64 one; one call of the
       // switch below for all three, so that its rounding does not depend on the source
-      float x0 = 0.f, x1 = 0.f, x2 = 0.f;
       bool have = false;
       if (g.disp) {
         if (dd.w > 0.5f) {  // FP32 r^2 certainly inside r_c
@@ -389,6 +438,8 @@ __global__ void __launch_bounds__(256, 3)
           have = fmaf(x0, x0, fmaf(x1, x1, x2 * x2)) < G->rc2_in;
         }
       }
+      if (NPASS == 3 && g.pos2)
+        have = two_float_disp(g, li, l2, j, nl_code[(long)i * pc.nc + k], frame_of(pc, i), x0, x1, x2);
       if (!have) {
         const int ie = g.disp ? g.perm[p] : i;
         if (g.disp) j = g.nl_j[(long)ie * pc.nc + k];
@@ -425,14 +476,6 @@ __global__ void __launch_bounds__(256, 3)
       } else {
         const unsigned vm = __ballot_sync(0xffffffffu, valid);
         if (vm) lmin = __shfl_sync(0xffffffffu, l, 31 - __clz(vm));
-      }
-    }
-    if (in) {
-      if (valid) {
-        g.envU[row] = make_float4(s, u[0], u[1], u[2]);
-        g.envB[row] = make_float4(ds, r, tau, __int_as_float(l));
-      } else {
-        g.envB[row] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
       }
     }
     // moments of this slot
@@ -489,7 +532,7 @@ __global__ void __launch_bounds__(256, 3)
     }
     // run index of every slot: runs so far + heads up to this lane - 1
     const int myrun = nruns + __popc(headmask & (0xffffffffu >> (31 - lane))) - 1;
-    if (valid) g.slot_run[row] = myrun;
+    if (valid) g.slot[row] = make_float4(x0, x1, x2, __int_as_float((myrun << 16) | l));
     // every run of the batch is complete except the one holding the last valid lane, unless
     // the list ends in this batch
     const int lastvalid = validmask ? 31 - __clz(validmask) : -1;
@@ -1215,6 +1258,7 @@ __global__ void __launch_bounds__(256)
   const int i = g.perm[p];
   float fi[3] = {0.f, 0.f, 0.f}, vir[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   const int* nlrow = g.nl_j + (long)i * pc.nc;
+  const float frs = (float)pc.rs, frc = (float)pc.rc, inv_w = 1.0f / (frc - frs);
   // (type, 32-slot batch) in order; the next batch's list entries are loaded before the current
   // batch is worked on, so one fewer dependent load is exposed per batch
   int t = 0, base = g.sel_off[0];
@@ -1239,10 +1283,13 @@ __global__ void __launch_bounds__(256)
       const int j = jc;
       if (j < 0) continue;
       const long row = (long)p * pc.nc + k;
-      const float4 e0 = g.envU[row], e1 = g.envB[row];
-      const long run = rbase + g.slot_run[row];
-      const float tau = e1.z;
-      const int l = __float_as_int(e1.w);
+      const float4 e = g.slot[row];
+      const unsigned rl = (unsigned)__float_as_int(e.w);
+      const long run = rbase + (rl >> 16);
+      const int l = rl & 0xFFFF;
+      float rr, s, ds, u[3];
+      pair_env_f32_fast(e.x, e.y, e.z, frs, frc, inv_w, rr, s, ds, u);
+      const float tau = tau_at(g, s, l);
       float gR[4], dg[4];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
@@ -1267,7 +1314,7 @@ __global__ void __launch_bounds__(256)
         gR[c] = P[0] + tau * (P[1] + tau * (P[2] + tau * (P[3] + tau * (P[4] + tau * P[5]))));
         dg[c] = P[1] + tau * (2.f * P[2] + tau * (3.f * P[3] + tau * (4.f * P[4] + tau * (5.f * P[5]))));
       }
-      const float s = e0.x, u0 = e0.y, u1 = e0.z, u2 = e0.w, ds = e1.x, rr = e1.y;
+      const float u0 = u[0], u1 = u[1], u2 = u[2];
       const float invd = l < g.n1 ? g.inv1 : g.inv2;
       const float gs = s * (dg[0] + u0 * dg[1] + u1 * dg[2] + u2 * dg[3]) * invd;
       const float gvu = gR[1] * u0 + gR[2] * u1 + gR[3] * u2;
@@ -1473,9 +1520,7 @@ int run_mom(const DeviceModel& m, const PathConst& pc, const PathIO& io, Arena& 
   __nv_bfloat16* D_lo = split_fit ? ar.get<__nv_bfloat16>(N * M * A) : nullptr;
   const long slots = N * pc.nc;
   const int parts = bf16 ? 1 : 2;
-  float4* envU = ar.get<float4>(slots);
-  float4* envB = ar.get<float4>(slots);
-  int* slot_run = ar.get<int>(slots);
+  float4* slot = ar.get<float4>(slots);
   const int ncl = (pc.nc + 7) & ~7;
   short* run_l = ar.get<short>(N * ncl);
   // (lists of more slots than the search keeps per type leave no room for the schedule's entries)
@@ -1531,10 +1576,10 @@ int run_mom(const DeviceModel& m, const PathConst& pc, const PathIO& io, Arena& 
   const int tiles = g.tile_start[pc.ntypes];
   g.perm = io.perm;
   g.nl_j = io.nl_j;
-  g.envU = envU;
-  g.envB = envB;
-  g.slot_run = slot_run;
+  g.slot = slot;
   g.run_l = run_l;
+  g.pos2 = io.pos2;
+  g.tshift2 = io.tshift2;
   g.ncl = ncl;
   g.run_mask = run_mask;
   g.run_rec = reinterpret_cast<uint4*>(runs);

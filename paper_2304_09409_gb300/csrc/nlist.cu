@@ -88,17 +88,29 @@ __device__ __forceinline__ Binned bin_atom(const NlGeom& g, const double* x) {
   return b;
 }
 
+// x as high and low floats: |x - (high + low)| <= 2^-48 |x|.
+__device__ __forceinline__ void store_two_float(const double* x, float4* out) {
+  float h[3], l[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    h[a] = (float)x[a];
+    l[a] = (float)(x[a] - (double)h[a]);
+  }
+  out[0] = make_float4(h[0], h[1], h[2], fmaxf(fabsf(h[0]), fmaxf(fabsf(h[1]), fabsf(h[2]))));
+  out[1] = make_float4(l[0], l[1], l[2], 0.f);
+}
+
 // Key (type, cell) of every atom, its rank among the atoms of that key (the count so far) and
 // its sorted entry (cell-local FP32 position with the atom index; image index m with the packed
 // cell coordinates).  When asked, the same launch also forms the 27 image translations
 // t(n) = n0 h0 + n1 h1 + n2 h2, n in {-1,0,1}^3, of every frame (rounded as the exact
-// displacement rounds them).
+// displacement rounds them), and positions and translations as two floats.
 __global__ void k_bin(const NlGeom* __restrict__ G, const int* __restrict__ atom_frame,
                       const int* __restrict__ cell_off, int natoms, int ncells_total, int ntypes,
                       const double* __restrict__ coord, const int* __restrict__ type, int* __restrict__ cell_count,
                       int2* __restrict__ atom_key, float4* __restrict__ atom_l, int4* __restrict__ atom_m,
                       DevStatus* __restrict__ st, const double* __restrict__ boxes, int nframes,
-                      double* __restrict__ tshift) {
+                      double* __restrict__ tshift, float4* __restrict__ pos2, float4* __restrict__ tshift2) {
   pdl_wait();
   pdl_next();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -107,9 +119,13 @@ __global__ void k_bin(const NlGeom* __restrict__ G, const int* __restrict__ atom
       const int f = k / 27, q = k - 27 * f;
       const double* h = boxes + 9L * f;
       const int n0 = q / 9 - 1, n1 = (q / 3) % 3 - 1, n2 = q % 3 - 1;
-      for (int a = 0; a < 3; ++a)
-        tshift[81L * f + q * 3 + a] = __dadd_rn(
-            __dadd_rn(__dmul_rn((double)n0, h[a]), __dmul_rn((double)n1, h[3 + a])), __dmul_rn((double)n2, h[6 + a]));
+      double t[3];
+      for (int a = 0; a < 3; ++a) {
+        t[a] = __dadd_rn(__dadd_rn(__dmul_rn((double)n0, h[a]), __dmul_rn((double)n1, h[3 + a])),
+                         __dmul_rn((double)n2, h[6 + a]));
+        tshift[81L * f + q * 3 + a] = t[a];
+      }
+      if (tshift2) store_two_float(t, tshift2 + 2L * k);
     }
   if (i >= natoms) return;
   const int fr = atom_frame ? atom_frame[i] : 0;
@@ -121,6 +137,7 @@ __global__ void k_bin(const NlGeom* __restrict__ G, const int* __restrict__ atom
     atomicExch(&st->bad_coord, 1);
     x[0] = x[1] = x[2] = 0.0;
   }
+  if (pos2) store_two_float(x, pos2 + 2L * i);
   const Binned b = bin_atom(g, x);
   const int t = type[i];
   if (t < 0 || t >= ntypes) {  // reported; the atom takes part in no list
@@ -1315,10 +1332,11 @@ cudaError_t launch_nlist_build(const NlLaunch& L, int ntypes, const double* coor
   std::memset(&nochk, 0, sizeof(nochk));
   const double* no_boxes = nullptr;
   double* no_tshift = nullptr;
+  float4* no_two = nullptr;
   e = launch_chain(L.pdl, k_bin, dim3((L.natoms + bin_threads - 1) / bin_threads), dim3(bin_threads), 0, st, L.geoms,
                    L.atom_frame, L.cell_off, L.natoms, L.ncells_total, ntypes, coord, type, cell_count, sc.atom_key,
                    sc.atom_l, sc.atom_m, status, ex ? ex->boxes : no_boxes, ex ? ex->nframes : 0,
-                   ex ? ex->tshift : no_tshift);
+                   ex ? ex->tshift : no_tshift, ex ? ex->pos2 : no_two, ex ? ex->tshift2 : no_two);
   if (e != cudaSuccess) return e;
   int* no_int = nullptr;
   if (nkeys <= 8192) {  // few keys: each fill block scans the counts itself (one launch fewer; nlist_launches)

@@ -182,6 +182,10 @@ struct PathIO {
   // from the cell-centred list build of this call (else null): [N][Nc] in sorted atom order, each
   // listed pair's FP32 displacement and, in w, 1 (FP32 usable), 0 (exact FP64 needed), -1 (padding)
   const float4* disp;
+  // from the list build of this call (else null): positions (input order) and image translations as
+  // two floats (NlExtras)
+  const float4* pos2;
+  const float4* tshift2;
 };
 
 struct __align__(32) D4 {
