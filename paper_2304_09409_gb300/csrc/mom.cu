@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(256, 3)
   int carry_l = -1;                          // interval of the run open at the last batch's end
   int nruns = 0;
   bool oor = false;
-  unsigned mask_lo = 0, mask_hi = 0;  // bit l >> 2 of the runs so far
+  unsigned mask_lo = 0, mask_hi = 0;  // bit l >> 2 of the lane's slots
   for (int base = kb0; base < kb1; base += 32) {
     const int k = base + lane;
     const bool in = k < kb1;
@@ -478,8 +478,25 @@ __global__ void __launch_bounds__(256, 3)
         if (vm) lmin = __shfl_sync(0xffffffffu, l, 31 - __clz(vm));
       }
     }
-    // moments of this slot
     const int lk = valid ? l : -2;
+    // run structure of the batch: a head starts a new run (the first lane may continue the run
+    // left open by the previous batch)
+    const int lprev_lane = __shfl_up_sync(0xffffffffu, lk, 1);
+    const int lprev = lane == 0 ? carry_l : lprev_lane;
+    const bool head = valid && lk != lprev;
+    const bool seg = valid && (lane == 0 || lk != lprev_lane);  // first lane of its run in this batch
+    const unsigned headmask = __ballot_sync(0xffffffffu, head);
+    const unsigned segmask = __ballot_sync(0xffffffffu, seg);
+    const unsigned validmask = __ballot_sync(0xffffffffu, valid);
+    // run index of every slot: runs so far + heads up to this lane - 1
+    const int myrun = nruns + __popc(headmask & (0xffffffffu >> (31 - lane))) - 1;
+    if (valid) g.slot[row] = make_float4(x0, x1, x2, __int_as_float((myrun << 16) | l));
+    if (g.run_mask) {
+      const int b = lk >> 2;
+      mask_lo |= valid && b < 32 ? 1u << b : 0u;
+      mask_hi |= valid && b >= 32 ? 1u << (b - 32) : 0u;
+    }
+    // moments of this slot
     float v[24];
     {
       const float R[4] = {s, s * u[0], s * u[1], s * u[2]};
@@ -491,15 +508,6 @@ __global__ void __launch_bounds__(256, 3)
         pw *= tau;
       }
     }
-    // run structure of the batch: a head starts a new run (the first lane may continue the run
-    // left open by the previous batch)
-    const int lprev_lane = __shfl_up_sync(0xffffffffu, lk, 1);
-    const int lprev = lane == 0 ? carry_l : lprev_lane;
-    const bool head = valid && lk != lprev;
-    const bool seg = valid && (lane == 0 || lk != lprev_lane);  // first lane of its run in this batch
-    const unsigned headmask = __ballot_sync(0xffffffffu, head);
-    const unsigned segmask = __ballot_sync(0xffffffffu, seg);
-    const unsigned validmask = __ballot_sync(0xffffffffu, valid);
     // segmented sums towards the first lane of each run; after the step of distance off every lane
     // holds the sum over its run up to 2 off - 1 lanes ahead, so once no run reaches off lanes
     // ahead the heads hold their runs' sums (runs are short: one to a few slots)
@@ -530,9 +538,6 @@ __global__ void __launch_bounds__(256, 3)
                            reinterpret_cast<unsigned char*>(dst + c * PARTS + 1), w8);
       }
     }
-    // run index of every slot: runs so far + heads up to this lane - 1
-    const int myrun = nruns + __popc(headmask & (0xffffffffu >> (31 - lane))) - 1;
-    if (valid) g.slot[row] = make_float4(x0, x1, x2, __int_as_float((myrun << 16) | l));
     // every run of the batch is complete except the one holding the last valid lane, unless
     // the list ends in this batch
     const int lastvalid = validmask ? 31 - __clz(validmask) : -1;
@@ -560,15 +565,14 @@ __global__ void __launch_bounds__(256, 3)
     }
     __syncwarp();
     nruns += __popc(headmask);
-    if (g.run_mask) {
-      const int b = lk >> 2;
-      mask_lo |= __reduce_or_sync(0xffffffffu, valid && b < 32 ? 1u << b : 0u);
-      mask_hi |= __reduce_or_sync(0xffffffffu, valid && b >= 32 ? 1u << (b - 32) : 0u);
-    }
     if (ends) break;  // warp-uniform: the rest of the block is padding
   }
   if (lane == 0 && nruns < kb1 - kb0) runl[nruns] = -1;
-  if (lane == 0 && g.run_mask) g.run_mask[task] = make_uint2(mask_lo, mask_hi);
+  if (g.run_mask) {
+    mask_lo = __reduce_or_sync(0xffffffffu, mask_lo);
+    mask_hi = __reduce_or_sync(0xffffffffu, mask_hi);
+    if (lane == 0) g.run_mask[task] = make_uint2(mask_lo, mask_hi);
+  }
   if (__any_sync(0xffffffffu, oor) && lane == 0) atomicOr(g.table_range, 1);
   }
 }
