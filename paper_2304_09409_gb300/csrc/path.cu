@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(kE3Warps * 32)
   V4* Rv = reinterpret_cast<V4*>(sm_raw);     // [nc] rows of the real neighbours, compacted
   V4* gRv = Rv + nc;                          // [nc] dE/dR of those rows (backward)
   R* wsm = reinterpret_cast<R*>(gRv + nc);    // [n_nets * per_net]
-  R* red = wsm + (long)n_nets * pn;           // [W] gD (backward)
+  R* red = wsm + (long)n_nets * pn;           // [W] D sums / gD
   int* tv = reinterpret_cast<int*>(red + W);  // [nc] neighbour type of each compacted row
   int* kv = tv + nc;                          // [nc] slot of each compacted row
   __shared__ int nv_s;
@@ -786,19 +786,14 @@ __global__ void __launch_bounds__(kE3Warps * 32)
   __syncwarp();
   if (oor && range_flag) atomicOr(range_flag, 1);
   if (!BWD) {
-    __shared__ R dsum[kE3Warps][W];
 #pragma unroll
     for (int m = 0; m < W; ++m) {
       R v = acc[m];
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) dsum[warp][m] = v;
+      if (lane == 0 && m < M) atomicAdd(&red[m], v);
     }
     __syncthreads();
-    if (tid < M) {  // the warps' sums in a fixed order, in FP64: D is the same from run to run
-      double d = 0.0;
-      for (int w = 0; w < nw; ++w) d += (double)dsum[w][tid];
-      D[(long)p * pc.Dw + pc.doff + tid] = R(d) * inv;
-    }
+    if (tid < M) D[(long)p * pc.Dw + pc.doff + tid] = red[tid] * inv;
   } else {
     __syncthreads();
     V4* out = reinterpret_cast<V4*>(gR) + rb;
