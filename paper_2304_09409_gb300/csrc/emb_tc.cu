@@ -546,6 +546,40 @@ __global__ void k_descr_bwd_b(PathConst pc, const float4* __restrict__ Tm, const
   }
 }
 
+// Adds the force and virial of a warp's pairs (one lane each; real: the lane has one) to their centre atoms:
+// gd to F_i, -gd d^T to the virial of i.  Neighbouring slots belong to one atom or two, so the lanes of each are
+// summed first (16 values by halving exchanges: 16 additions, not 60) and twelve lanes add the sums.  With twelve
+// FP64 atomics a pair, all to one atom's lines, they bound the kernel (8,736 atoms of 512 slots: 498 -> 391 us; the
+// CUDA-core path's force kernel, whose FP64 pipe is as busy, gained nothing from it: 136 -> 157 us).
+// p: the lane's sorted atom, i its index.  Every lane of the warp calls it.
+__device__ __forceinline__ void add_to_centre(bool real, int p, int i, const double* gd, const double* d,
+                                              double* __restrict__ force, double* __restrict__ avir) {
+  const int lane = threadIdx.x & 31;
+  unsigned todo = __ballot_sync(0xffffffffu, real);
+  while (todo) {
+    const int src = __ffs(todo) - 1;
+    const int p0 = __shfl_sync(0xffffffffu, p, src), i0 = __shfl_sync(0xffffffffu, i, src);
+    const bool mine = real && p == p0;
+    double v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+      v[q] = !mine || q >= 12 ? 0.0 : (q < 3 ? gd[q < 3 ? q : 0] : -gd[q >= 3 ? (q - 3) / 3 % 3 : 0] * d[q % 3]);
+#pragma unroll
+    for (int h = 8; h > 0; h >>= 1) {
+      const bool up = lane & (2 * h);
+#pragma unroll
+      for (int q = 0; q < h; ++q) {
+        const double send = up ? v[q] : v[q + h], keep = up ? v[q + h] : v[q];
+        v[q] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * h);
+      }
+    }
+    const double sum = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+    const int q = lane >> 1;
+    if (!(lane & 1) && q < 12) atomicAdd(q < 3 ? force + 3L * i0 + q : avir + 9L * i0 + (q - 3), sum);
+    todo &= ~__ballot_sync(0xffffffffu, mine);
+  }
+}
+
 // Backward of the scalar first layer (dE/ds from dE/dy0), then dE/dr_ij and the FP64 force and
 // virial scatter.
 __global__ void __launch_bounds__(256)
@@ -555,44 +589,44 @@ __global__ void __launch_bounds__(256)
                    const float* __restrict__ T0, const float4* __restrict__ gR, double* __restrict__ force,
                    double* __restrict__ avir) {
   const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long)pc.natoms * pc.nc) return;
-  const int p = (int)(e / pc.nc), k = (int)(e % pc.nc);
-  const int i = perm[p];
-  const int j = nl_j[(long)i * pc.nc + k];
-  if (j < 0) return;
-  const int t = block_of_slot(pc, k);
-  const long row = brow(pc, p, k, t);
-  const int net = pc.type_one_side ? t : tsorted[p] * pc.ntypes + t;
-  const float* w = nets.w0[net];
-  double d[3];
-  listed_disp(coord + 3 * i, coord + 3 * j, nl_code[(long)i * pc.nc + k], pc, frame_of(pc, i), d[0], d[1], d[2]);
-  float r, s, ds, u[3];
-  pair_env<float>(d[0], d[1], d[2], norm2_exact(d[0], d[1], d[2]), pc.rs, pc.rc, pc.near2, r, s, ds, u);
-  // a pair whose s rounded to zero (within ~1e-15 of r_c) had no layer epilogues: its rows are not
-  // read, and its force terms (s = 0, |ds/dr| below 1e-29) are zero
-  if (s == 0.f) return;
-  float gs = 0.f;
-  for (int c = 0; c < w1; ++c) {
-    const float gy = G0[row * ld1 + c], tt = T0[row * ld1 + c];
-    gs += gy * (1.f - tt * tt) * __ldg(w + c);
-    if (skip) gs += gy;
+  double d[3] = {0.0, 0.0, 0.0}, gd[3] = {0.0, 0.0, 0.0};
+  int p = -1, i = -1;
+  bool real = false;
+  if (e < (long)pc.natoms * pc.nc) {
+    p = (int)(e / pc.nc);
+    const int k = (int)(e % pc.nc);
+    i = perm[p];
+    const int j = nl_j[(long)i * pc.nc + k];
+    if (j >= 0) {
+      listed_disp(coord + 3 * i, coord + 3 * j, nl_code[(long)i * pc.nc + k], pc, frame_of(pc, i), d[0], d[1], d[2]);
+      float r, s, ds, u[3];
+      pair_env<float>(d[0], d[1], d[2], norm2_exact(d[0], d[1], d[2]), pc.rs, pc.rc, pc.near2, r, s, ds, u);
+      // a pair whose s rounded to zero (within ~1e-15 of r_c) had no layer epilogues: its rows are not
+      // read, and its force terms (s = 0, |ds/dr| below 1e-29) are zero
+      if (s != 0.f) {
+        real = true;
+        const int t = block_of_slot(pc, k);
+        const long row = brow(pc, p, k, t);
+        const int net = pc.type_one_side ? t : tsorted[p] * pc.ntypes + t;
+        const float* w = nets.w0[net];
+        float gs = 0.f;
+        for (int c = 0; c < w1; ++c) {
+          const float gy = G0[row * ld1 + c], tt = T0[row * ld1 + c];
+          gs += gy * (1.f - tt * tt) * __ldg(w + c);
+          if (skip) gs += gy;
+        }
+        const float4 g4 = gR[row];
+        const float gvu = g4.y * u[0] + g4.z * u[1] + g4.w * u[2];
+        const float a = ds * (gs + g4.x + gvu), b = s / r;
+        const float gv[3] = {g4.y, g4.z, g4.w};
+#pragma unroll
+        for (int c = 0; c < 3; ++c) gd[c] = (double)(a * u[c] + b * (gv[c] - gvu * u[c]));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) atomicAdd(force + 3 * j + c, -gd[c]);
+      }
+    }
   }
-  const float4 g4 = gR[row];
-  const float gvu = g4.y * u[0] + g4.z * u[1] + g4.w * u[2];
-  const float a = ds * (gs + g4.x + gvu), b = s / r;
-  const float gv[3] = {g4.y, g4.z, g4.w};
-  double gd[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) gd[c] = (double)(a * u[c] + b * (gv[c] - gvu * u[c]));
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    atomicAdd(force + 3 * i + c, gd[c]);
-    atomicAdd(force + 3 * j + c, -gd[c]);
-  }
-#pragma unroll
-  for (int aa = 0; aa < 3; ++aa)
-#pragma unroll
-    for (int bb = 0; bb < 3; ++bb) atomicAdd(avir + 9L * i + aa * 3 + bb, -gd[aa] * d[bb]);
+  add_to_centre(real, p, i, gd, d, force, avir);
 }
 
 __global__ void k_types_of_sorted(const int* __restrict__ type, const int* __restrict__ perm, int n,
