@@ -179,15 +179,15 @@ def _candidate_pairs(frame, rc):
 def _kernel_rooflines(cfg, big, real_nb, prof, work, steps, peaks, fit_npass):
     """Roofline of each timed scope.  Work per launch:
       nlist      HBM: coordinates and type in (28 B/atom), list and image code out (8 B/slot)
-      env        HBM: the list build's FP32 displacement read 16 B/slot, (ds, r, tau, l) 16 B/slot,
-                 (s, u) 16 B + run index 4 B per real neighbour (run moment records not counted)
+      env        HBM: index and image code read 8 B, displacement and run written 16 B per real neighbour
+                 (run moment records not counted)
       mom_fwd    tensor: the MMA FLOPs the kernel issued (2 x 128 rows x padded M x 64 per K block
                  and pass, counted on the device), against the BF16/FP16 dense peak; the FP32-ALU
                  equivalent of the paper's per-neighbour Horner loop (18 M FLOP per real
                  neighbour) is kept as a side figure
       mom_bwd    tensor: issued MMA FLOPs as mom_fwd (side figure 36 M FLOP per real neighbour)
       mom_gT     HBM: dE/dD read 4 M M_< B/atom (2 B in the mixed mode), T and T_< 16 (M + M_<) B/atom
-      mom_force  HBM: env rows 32 B + run index 4 B per real neighbour, run P 32 B per real
+      mom_force  HBM: pair record 16 B + index 4 B per real neighbour, run P 32 B per real
                  neighbour (upper bound of runs), force and virial 96 B/atom
       fit_*      tensor: 2 rows K N per GEMM of the scope (fit_fused_tc: the whole net, both ways),
                  times the passes the path issues (3 for the split operands of the FP32 mode)
@@ -206,9 +206,9 @@ def _kernel_rooflines(cfg, big, real_nb, prof, work, steps, peaks, fit_npass):
     dd_bytes = 2 if fit_npass == 1 else 4
     work_tab = {
         "nlist": ("hbm", (N * 28 + N * nc * 8) / 1e9, hbm, "GB/s"),
-        "env": ("hbm", (N * nc * 32 + real_nb * 20) / 1e9, hbm, "GB/s"),
+        "env": ("hbm", real_nb * 24 / 1e9, hbm, "GB/s"),
         "mom_gT": ("hbm", (N * (dd_bytes * M * A + 16 * (M + A))) / 1e9, hbm, "GB/s"),
-        "mom_force": ("hbm", (real_nb * 68 + N * 96) / 1e9, hbm, "GB/s"),
+        "mom_force": ("hbm", (real_nb * 52 + N * 96) / 1e9, hbm, "GB/s"),
         "fit_fwd_tc": ("tensor", fit_npass * fwd / 1e12, ten, "TFLOP/s"),
         "fit_fwd_last_tc": ("tensor", fit_npass * fwd_last / 1e12, ten, "TFLOP/s"),
         "fit_bwd_tc": ("tensor", fit_npass * bwd / 1e12, ten, "TFLOP/s"),

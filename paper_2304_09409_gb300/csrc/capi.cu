@@ -203,9 +203,10 @@ int read_status(dp_model* md, cudaStream_t st, int* n_overflow) {
   md->prof.collect();
   const DevStatus s = *md->status_host;
   if (md->prof.timing && md->m.mom_npass) {  // issued MMA work of the moment kernels
-    // one block: 128 accumulator rows x 64 x the padded width M, times the passes
+    // one block: 128 accumulator rows x 64 x the padded width M, times the passes (the three-pass forward's
+    // blocks are 32 wide)
     const double per = 2.0 * 128.0 * 64.0 * md->m.mom_npad * md->m.mom_npass;
-    if (s.mma_blocks[0]) md->prof.work[md->prof.id_of("mom_fwd")] += per * s.mma_blocks[0];
+    if (s.mma_blocks[0]) md->prof.work[md->prof.id_of("mom_fwd")] += (md->m.mom_npass == 3 ? 0.5 : 1.0) * per * s.mma_blocks[0];
     if (s.mma_blocks[1]) md->prof.work[md->prof.id_of("mom_bwd")] += per * s.mma_blocks[1];
   }
   if (n_overflow) *n_overflow = s.sel_overflow;
