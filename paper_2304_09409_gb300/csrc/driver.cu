@@ -455,7 +455,8 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
       if (!gr) {
         clear(host_f ? b.force : force, sizeof(double) * 3 * N);
         clear(b.fcount, sizeof(int) * F);
-        if (!m.compressed) clear(b.atom_virial, sizeof(double) * 9 * N);
+        // the compressed se_e2_a kernels write every atom's virial, every other path adds to it pair by pair
+        if (!(m.compressed && m.cfg.descriptor == DP_DESC_SE_E2_A)) clear(b.atom_virial, sizeof(double) * 9 * N);
       }
       ProfScope _ps(&md->prof, "clear", s);
       k_clear<<<(unsigned)std::min<long>((most + 255) / 256, 4L * sm_count()), 256, 0, s>>>(ca);
