@@ -266,7 +266,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / 4))
   int gi = 0;
   while (gi + 1 < g.rows.ngroups && tile >= g.tile0[gi + 1]) ++gi;
   const DenseGroup grp = g.rows.g[gi];
-  const int nrows = g.rows.list ? __ldg(g.rows.count + gi) : grp.nrows;
+  const int nrows = g.rows.rows_of(gi);
   const int r0 = (tile - g.tile0[gi]) * BM;
   if (r0 >= nrows) return;  // the whole cluster leaves: the rows do not depend on cr
   for (int r = tid; r < BM; r += NT) {
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / 4))
     int at = 0;
     for (int k = 0; k < ng; ++k) {
       s_tile0[k] = at;
-      at += ((g.rows.list ? __ldg(g.rows.count + k) : g.rows.g[k].nrows) + BM - 1) / BM;
+      at += (g.rows.rows_of(k) + BM - 1) / BM;
     }
     s_tile0[ng] = at;
   }
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / 4))
     if (tid >= BM || tile >= t1) return -1;
     const int k = group_of(tile);
     const DenseGroup& grp = g.rows.g[k];
-    const int nrows = g.rows.list ? __ldg(g.rows.count + k) : grp.nrows;
+    const int nrows = g.rows.rows_of(k);
     const int r = (tile - s_tile0[k]) * BM + tid;
     if (r >= nrows) return -1;
     return g.rows.list ? __ldg(g.rows.list + grp.r0 + r) : (int)grp.r0 + r;

@@ -19,22 +19,32 @@ struct DenseRows {
   const int* count = nullptr;  // device [ngroups], list mode only
   DenseGroup g[kMaxDenseGroups];
   void add(long r0, int nrows, long w) { g[ngroups++] = DenseGroup{r0, w, nrows}; }
+  // rows of group k; a list holds at most nrows entries whatever was counted (append_row)
+  __device__ __forceinline__ int rows_of(int k) const {
+    return list ? min(__ldg(count + k), g[k].nrows) : g[k].nrows;
+  }
 };
 
 // Row lists of a descriptor part: the slot rows with s != 0 (the others are padding) of every
 // (centre type, neighbour type) pair, compacted so that no layer works on padding.  Entries of pair
-// (ti, tj) start at base[ti * ntypes + tj]; their order within a pair is arbitrary.
+// (ti, tj) start at base[ti * ntypes + tj], and there is room for cap[ti * ntypes + tj] of them; their
+// order within a pair is arbitrary.
+// The room follows the per-type counts the call was set up with.  A device type array may have been rewritten
+// since those were read: that is found on the device and the call is done again, but its kernels run to the
+// end first, so entries beyond a pair's room are dropped.
 struct RowLists {
   int* list = nullptr;
   int* count = nullptr;
   long base[kMaxDenseGroups];
+  int cap[kMaxDenseGroups];
 };
 
-// Append every calling thread's row (grp >= 0) to its group's list; the whole block calls.  One global
-// atomic per block and group.
+// Append every calling thread's row (grp in [0, ngroups)) to its group's list; the whole block calls.  One
+// global atomic per block and group.
 __device__ __forceinline__ void append_row(const RowLists& rl, int ngroups, int grp, long row) {
   __shared__ int s_cnt[kMaxDenseGroups], s_base[kMaxDenseGroups];
   for (int e = threadIdx.x; e < ngroups; e += blockDim.x) s_cnt[e] = 0;
+  if (grp >= ngroups) grp = -1;
   __syncthreads();
   const unsigned lane = threadIdx.x & 31u;
   const unsigned peers = __match_any_sync(0xffffffffu, grp);
@@ -46,7 +56,7 @@ __device__ __forceinline__ void append_row(const RowLists& rl, int ngroups, int 
   for (int e = threadIdx.x; e < ngroups; e += blockDim.x)
     if (s_cnt[e] > 0) s_base[e] = atomicAdd(rl.count + e, s_cnt[e]);
   __syncthreads();
-  if (grp >= 0) rl.list[rl.base[grp] + s_base[grp] + at] = (int)row;
+  if (grp >= 0 && s_base[grp] + at < rl.cap[grp]) rl.list[rl.base[grp] + s_base[grp] + at] = (int)row;
 }
 
 // Row stride of the activations of an inner layer of width w: whole 16-byte (FP32) or 32-byte (FP64)

@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kWgThreads)
   int gi = 0;
   while (gi + 1 < g.rows.ngroups && (int)blockIdx.z >= g.slab0[gi + 1]) ++gi;
   const DenseGroup grp = g.rows.g[gi];
-  const int nrows = g.rows.list ? __ldg(g.rows.count + gi) : grp.nrows;
+  const int nrows = g.rows.rows_of(gi);
   const int rbeg = ((int)blockIdx.z - g.slab0[gi]) * g.slab_rows[gi];
   const int rend = min(nrows, rbeg + g.slab_rows[gi]);
   if (rbeg >= rend) return;
@@ -492,7 +492,8 @@ int run_grad(const DeviceModel& m, const PathConst& pc, const R* params, const P
   for (int ti = 0; ti < nt; ++ti)
     for (int tj = 0; tj < nt; ++tj) {
       lists.base[ti * nt + tj] = list_at;
-      list_at += (long)(io.type_start[ti + 1] - io.type_start[ti]) * pc.sel[tj];
+      lists.cap[ti * nt + tj] = (io.type_start[ti + 1] - io.type_start[ti]) * pc.sel[tj];
+      list_at += lists.cap[ti * nt + tj];
     }
   if (ar.measure) return DP_OK;
   if (!ar.ok()) {

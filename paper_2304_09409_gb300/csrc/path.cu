@@ -1268,7 +1268,8 @@ int run_generic(const DeviceModel& m, const PathConst& pc, const R* params, cons
     for (int ti = 0; ti < pc.ntypes; ++ti)
       for (int tj = 0; tj < pc.ntypes; ++tj) {
         b.lists.base[ti * pc.ntypes + tj] = at;
-        at += (long)(io.type_start[ti + 1] - io.type_start[ti]) * P.sel[tj];
+        b.lists.cap[ti * pc.ntypes + tj] = (io.type_start[ti + 1] - io.type_start[ti]) * P.sel[tj];
+        at += b.lists.cap[ti * pc.ntypes + tj];
       }
   }
   R* D = ar.get<R>(N * pc.Dw);
