@@ -212,6 +212,10 @@ inline cudaError_t allow_max_smem(K kernel) {
   return e;
 }
 
+// Type of an atom for indexing: one outside [0, ntypes) counts as type 0.  The list build reports it and the call
+// fails with DP_E_ARG, but (device types, known after the call only) its kernels run to the end first.
+__device__ __forceinline__ int type_in_range(int t, int ntypes) { return (unsigned)t < (unsigned)ntypes ? t : 0; }
+
 // ------------------------------------------------------------------------------------------
 // Launchers (nlist.cu)
 // ------------------------------------------------------------------------------------------

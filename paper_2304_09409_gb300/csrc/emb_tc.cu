@@ -629,10 +629,10 @@ __global__ void __launch_bounds__(256)
   add_to_centre(real, p, i, gd, d, force, avir);
 }
 
-__global__ void k_types_of_sorted(const int* __restrict__ type, const int* __restrict__ perm, int n,
+__global__ void k_types_of_sorted(const int* __restrict__ type, const int* __restrict__ perm, int n, int ntypes,
                                   int* __restrict__ out) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < n) out[p] = type[perm[p]];
+  if (p < n) out[p] = type_in_range(type[perm[p]], ntypes);
 }
 
 unsigned nblk(long n, int b) { return (unsigned)((n + b - 1) / b); }
@@ -819,7 +819,7 @@ int run_tc_impl(const DeviceModel& m, const PathConst& pc0, const PathIO& io, Ar
   // ---- forward: R and the first layer, then the GEMM layers of the embedding ----
   {
     ProfScope _ps(io.prof, "sorted_types", st);
-    k_types_of_sorted<<<nblk(N, 256), 256, 0, st>>>(io.type, io.perm, (int)N, tsorted);
+    k_types_of_sorted<<<nblk(N, 256), 256, 0, st>>>(io.type, io.perm, (int)N, pc.ntypes, tsorted);
   }
   NetPtrs<float> nets;
   for (int n = 0; n < m.n_embed_nets; ++n) {

@@ -377,10 +377,10 @@ __global__ void k_to_double(const R* __restrict__ x, long n, double* __restrict_
   if (e < n) y[e] = (double)x[e];
 }
 
-__global__ void k_types_sorted(const int* __restrict__ type, const int* __restrict__ perm, int n,
+__global__ void k_types_sorted(const int* __restrict__ type, const int* __restrict__ perm, int n, int ntypes,
                                int* __restrict__ out, int* __restrict__ row_count) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < n) out[p] = type[perm[p]];
+  if (p < n) out[p] = type_in_range(type[perm[p]], ntypes);
   if (p < kMaxDenseGroups) row_count[p] = 0;
 }
 
@@ -501,7 +501,7 @@ int run_grad(const DeviceModel& m, const PathConst& pc, const R* params, const P
     return DP_E_OOM;
   }
   k_zero<R><<<nb(m.n_params, 256), 256, 0, st>>>(grad, m.n_params);
-  k_types_sorted<<<nb(N, 256), 256, 0, st>>>(io.type, io.perm, (int)N, tsorted, lists.count);
+  k_types_sorted<<<nb(N, 256), 256, 0, st>>>(io.type, io.perm, (int)N, nt, tsorted, lists.count);
   // ---- forward: primal and tangent ----
   {
     ProfScope _ps(io.prof, "grad_env", st);

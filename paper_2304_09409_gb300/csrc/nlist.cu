@@ -104,13 +104,15 @@ __device__ __forceinline__ void store_two_float(const double* x, float4* out) {
 // its sorted entry (cell-local FP32 position with the atom index; image index m with the packed
 // cell coordinates).  When asked, the same launch also forms the 27 image translations
 // t(n) = n0 h0 + n1 h1 + n2 h2, n in {-1,0,1}^3, of every frame (rounded as the exact
-// displacement rounds them), and positions and translations as two floats.
+// displacement rounds them), and positions and translations as two floats.  whole: the keys become the path's
+// type-sorted order, which has to hold every atom, one of no valid type among those of type 0.
 __global__ void k_bin(const NlGeom* __restrict__ G, const int* __restrict__ atom_frame,
                       const int* __restrict__ cell_off, int natoms, int ncells_total, int ntypes,
                       const double* __restrict__ coord, const int* __restrict__ type, int* __restrict__ cell_count,
                       int2* __restrict__ atom_key, float4* __restrict__ atom_l, int4* __restrict__ atom_m,
                       DevStatus* __restrict__ st, const double* __restrict__ boxes, int nframes,
-                      double* __restrict__ tshift, float4* __restrict__ pos2, float4* __restrict__ tshift2) {
+                      double* __restrict__ tshift, float4* __restrict__ pos2, float4* __restrict__ tshift2,
+                      bool whole) {
   pdl_wait();
   pdl_next();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -139,11 +141,13 @@ __global__ void k_bin(const NlGeom* __restrict__ G, const int* __restrict__ atom
   }
   if (pos2) store_two_float(x, pos2 + 2L * i);
   const Binned b = bin_atom(g, x);
-  const int t = type[i];
-  if (t < 0 || t >= ntypes) {  // reported; the atom takes part in no list
-    atom_key[i] = make_int2(-1, 0);
+  const int t = type_in_range(type[i], ntypes);
+  if (t != type[i]) {  // reported
     atomicExch(&st->bad_type, 1);
-    return;
+    if (!whole) {  // the atom takes part in no list
+      atom_key[i] = make_int2(-1, 0);
+      return;
+    }
   }
   const int key = t * ncells_total + (cell_off ? cell_off[fr] : 0) + (b.c[0] * g.ncell[1] + b.c[1]) * g.ncell[2] + b.c[2];
   atom_key[i] = make_int2(key, atomicAdd(cell_count + key, 1));
@@ -1097,8 +1101,8 @@ __global__ void __launch_bounds__(1024)
   for (int t = 0; t < DP_MAX_TYPES; ++t) cnt[t] = 0;
   bool bad = false;
   for (int i = lo; i < hi; ++i) {
-    const int t = type[i];
-    if (t < 0 || t >= ntypes) bad = true;
+    const int t = type_in_range(type[i], ntypes);
+    if (t != type[i]) bad = true;
 #pragma unroll
     for (int q = 0; q < DP_MAX_TYPES; ++q) cnt[q] += (t == q);
   }
@@ -1132,7 +1136,7 @@ __global__ void __launch_bounds__(1024)
 #pragma unroll
   for (int t = 0; t < DP_MAX_TYPES; ++t) off[t] = (t < ntypes) ? tstart[t] + wtot[w][t] + incl[t] - cnt[t] : 0;
   for (int i = lo; i < hi; ++i) {
-    const int t = type[i];
+    const int t = type_in_range(type[i], ntypes);
 #pragma unroll
     for (int q = 0; q < DP_MAX_TYPES; ++q)
       if (t == q && q < ntypes) perm[off[q]++] = i;
@@ -1336,7 +1340,7 @@ cudaError_t launch_nlist_build(const NlLaunch& L, int ntypes, const double* coor
   e = launch_chain(L.pdl, k_bin, dim3((L.natoms + bin_threads - 1) / bin_threads), dim3(bin_threads), 0, st, L.geoms,
                    L.atom_frame, L.cell_off, L.natoms, L.ncells_total, ntypes, coord, type, cell_count, sc.atom_key,
                    sc.atom_l, sc.atom_m, status, ex ? ex->boxes : no_boxes, ex ? ex->nframes : 0,
-                   ex ? ex->tshift : no_tshift, ex ? ex->pos2 : no_two, ex ? ex->tshift2 : no_two);
+                   ex ? ex->tshift : no_tshift, ex ? ex->pos2 : no_two, ex ? ex->tshift2 : no_two, ex && ex->perm);
   if (e != cudaSuccess) return e;
   int* no_int = nullptr;
   if (nkeys <= 8192) {  // few keys: each fill block scans the counts itself (one launch fewer; nlist_launches)

@@ -898,10 +898,10 @@ __global__ void k_shift_table(PathConst pc, double* __restrict__ out) {
 }
 
 // Types in sorted order; also clears the row-list counters (before the kernels that fill the lists).
-__global__ void k_sorted_types(const int* __restrict__ type, const int* __restrict__ perm, int n,
+__global__ void k_sorted_types(const int* __restrict__ type, const int* __restrict__ perm, int n, int ntypes,
                                int* __restrict__ out, int* __restrict__ row_count, int ncount) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < n) out[p] = type[perm[p]];
+  if (p < n) out[p] = type_in_range(type[perm[p]], ntypes);
   if (p < ncount) row_count[p] = 0;
 }
 
@@ -1284,7 +1284,7 @@ int run_generic(const DeviceModel& m, const PathConst& pc, const R* params, cons
   }
   {
     ProfScope _ps(io.prof, "sorted_types", st);
-    k_sorted_types<<<nblk(N, 256), 256, 0, st>>>(io.type, io.perm, (int)N, tsorted, row_count,
+    k_sorted_types<<<nblk(N, 256), 256, 0, st>>>(io.type, io.perm, (int)N, pc.ntypes, tsorted, row_count,
                                                   nparts * kMaxDenseGroups);
   }
   // ---- forward, part by part ----

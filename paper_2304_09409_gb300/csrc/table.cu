@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(128)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int p = blockIdx.x * 4 + warp;
   if (p >= pc.natoms) return;
-  const int i = perm[p], ti = type[i];
+  const int i = perm[p], ti = type_in_range(type[i], pc.ntypes);
   const int M = pc.M, nc = pc.nc, A = pc.A;
   R acc[MPL][4];
 #pragma unroll
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
   for (int q = 0; q < 9; ++q) v[q] = R(0);
   if (p < pc.natoms) {
-    const int i = perm[p], ti = type[i];
+    const int i = perm[p], ti = type_in_range(type[i], pc.ntypes);
     for (int e = lane; e < M * 4; e += 32) Ts[e] = Tm[(long)p * M * 4 + e];
     __syncwarp();
     // dE/dT[m][c] = sum_l dE/dD[m][l] T[l][c] + [m < M_<] sum_q dE/dD[q][m] T[q][c]
