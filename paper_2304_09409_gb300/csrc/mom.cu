@@ -121,7 +121,8 @@ __device__ __forceinline__ int mom_interval(const MomArgs& g, float s, int lcap,
     l = (int)floorf((s - g.s0) * g.inv1);
     l = l < 0 ? 0 : (l > g.n1 - 1 ? g.n1 - 1 : l);
   } else {
-    l = g.n1 + (int)floorf((s - g.split) * g.inv2);
+    // (the conversion saturates: a pair nearer than about 1e-9 A must not wrap the sum)
+    l = g.n1 + min((int)floorf((s - g.split) * g.inv2), g.lc);
     if (l > g.lc - 1) l = g.lc - 1;
     if (s > g.smax) oor = true;
   }

@@ -66,7 +66,7 @@ __device__ __forceinline__ int tab_interval(const TabConst& tc, R s, R& tt, bool
     l = l < 0 ? 0 : (l > tc.n1 - 1 ? tc.n1 - 1 : l);
     tt = s - (R(tc.s0) + R(l) * R(tc.stride1));
   } else {
-    l = tc.n1 + (int)floor((s - R(tc.split)) * R(1.0 / tc.stride2));
+    l = tc.n1 + min((int)floor((s - R(tc.split)) * R(1.0 / tc.stride2)), tc.lc);  // the conversion saturates
     if (l > tc.lc - 1) l = tc.lc - 1;
     tt = s - (R(tc.split) + R(l - tc.n1) * R(tc.stride2));
     if (s > R(tc.smax)) oor = true;
