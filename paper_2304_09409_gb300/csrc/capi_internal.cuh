@@ -22,9 +22,10 @@ struct dp_model {
   unsigned char* stage = nullptr;          // pinned staging for small per-call uploads
   size_t stage_cap = 0;
   dpgb::Prof prof;
-  // set once a frame overflowed the density-sized candidate buffer: later builds use the
-  // full DP_MAX_CANDIDATES buffer
-  bool nl_full_cap = false;
+  // Size of the neighbour search, raised for good when a frame (of uneven density) overflows it: 0 buffers
+  // by the mean density, half-width cells allowed; 1 whole cells and buffers of 512 entries, the largest of
+  // the cell-centred search; 2 DP_MAX_CANDIDATES, the per-atom search
+  int nl_step = 0;
   // per-type atom counts of the last device type array seen (checked on the device when reused)
   const int* ts_ptr = nullptr;
   int ts_n = -1;

@@ -192,10 +192,10 @@ int build_tables_host(dp_model* md, int F, const int* natoms, const double* boxe
   T.cap = 0;
   for (int f = 0; f < F; ++f) {
     const int rc = host_geometry(md->m.lcfg, natoms[f], boxes ? boxes + 9 * f : nullptr, lohi, T.geoms[f],
-                                  !(md->m.compressed && md->m.mom_npass == 1));
+                                  md->nl_step == 0 && !(md->m.compressed && md->m.mom_npass == 1));
     if (rc != DP_OK) return rc;
     NlGeom& g = T.geoms[f];
-    if (md->nl_full_cap) g.cap = DP_MAX_CANDIDATES;
+    if (md->nl_step) g.cap = md->nl_step == 1 ? std::max(g.cap, 512) : DP_MAX_CANDIDATES;
     T.cap = std::max(T.cap, g.cap);
     T.cell_off[f + 1] = T.cell_off[f] + g.ncell[0] * g.ncell[1] * g.ncell[2];
     if (boxes)
@@ -555,8 +555,8 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
       drop_graph(md);
       return run_frames(md, nlist, F, natoms, coord, type, boxes, energy, force, virial, atom_energy, st, gr);
     }
-    if (r == DP_E_CAPACITY && own_nlist && !md->nl_full_cap) {
-      md->nl_full_cap = true;  // retry once with the full candidate buffer
+    if (r == DP_E_CAPACITY && own_nlist && md->nl_step < 2) {
+      ++md->nl_step;  // retry with the next larger search
       drop_graph(md);
       return run_frames(md, nlist, F, natoms, coord, type, boxes, energy, force, virial, atom_energy, st, gr);
     }
@@ -591,7 +591,7 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
       sig.push_back(u);
     }
     for (int t = 0; t <= m.cfg.ntypes; ++t) sig.push_back((unsigned long long)(unsigned)chk.v[t]);
-    sig.push_back((unsigned long long)md->nl_full_cap | ((unsigned long long)md->prof.timing << 1));
+    sig.push_back((unsigned long long)md->nl_step | ((unsigned long long)md->prof.timing << 2));
     sig.push_back((unsigned long long)(copy_coord | (copy_type << 1) | (host_e << 2) | (host_v << 3) |
                                        (host_f << 4) | (dev_ae << 5)));
   }
@@ -797,8 +797,8 @@ int dp_build_nlist(dp_model* md, int N, const double* coord, const int* type, co
   rc = read_status(md, st, n_overflow);
   if (rc != DP_OK && rc != DP_E_SEL_OVERFLOW) {
     dp_free_nlist(nl);
-    if (rc == DP_E_CAPACITY && !md->nl_full_cap) {
-      md->nl_full_cap = true;  // retry once with the full candidate buffer
+    if (rc == DP_E_CAPACITY && md->nl_step < 2) {
+      ++md->nl_step;  // retry with the next larger search
       return dp_build_nlist(md, N, coord, type, box, out, n_overflow, stream);
     }
     return rc;

@@ -783,7 +783,7 @@ __global__ void __launch_bounds__(kCellWarps * 32, CAP <= 256 ? 4 : 3)
   const int P = s_tpex[ntypes];
   const int nce = s_cpre[ntypes];
   if (P > S) {  // CTA-uniform: the stream does not fit the staging buffer.  The call reports it
-                // (and is retried on the per-atom kernel); meanwhile this cell's rows are left
+                // (and is retried with a larger search); meanwhile this cell's rows are left
                 // empty, so that the kernels after the list stay in bounds.
     if (tid == 0) atomicExch(&st->capacity, 1);
     for (int q = warp; q < nce && blockIdx.y == 0; q += kCellWarps) {
@@ -1361,7 +1361,8 @@ cudaError_t launch_nlist_build(const NlLaunch& L, int ntypes, const double* coor
   const int ccap = std::min(L.cap <= 128 ? 128 : std::max(256, (L.cap + 63) & ~63), 1024);  // the cell kernel's
   // cell-centred search, one CTA per cell, when a cell's candidate stream fits shared memory:
   // room for 1.25 times the mean stream of a cell plus each type's padding (a cell with more
-  // reports a capacity error, and the call is retried on the per-atom kernel below)
+  // reports a capacity error, as does a denser group of one type than the buffer holds, and the call is
+  // retried with whole cells and the largest buffer, then on the per-atom kernel below)
   const double mean_stream = L.max_stream > 0 ? (double)L.max_stream
                                               : (double)L.natoms / std::max(1, L.ncells_total) * std::max(1, L.max_noff);
   const int S = std::max(1024, ((int)(1.25 * mean_stream) + 64 * ntypes + 64 + 127) & ~127);

@@ -1,0 +1,93 @@
+"""Frames of uneven density, which overflow a neighbour search sized by the mean density: a dense blob (more
+neighbours of one type than the buffer that the mean asks for), a rod in a box of 1.9 cutoffs (half-width cells whose
+stream is longer than the mean by more than the margin).  Integer results, bit-exact against the oracle's brute-force
+list, in the first call, which is retried, and in the next; and neither ends on the search for the largest buffer.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2304_09409_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+CFG = I.ModelConfig(ntypes=1, rcut=8.0, rcut_smth=0.5, sel=(512,), embed=(8, 16, 32), axis=4, fit=(32, 32))
+
+
+def _scatter(rng, box, n, draw, pts, apart):
+    """pts and n more points, no two nearer than apart (cubic box)."""
+    while n:
+        x = draw(rng)
+        d = np.array(pts).reshape(-1, 3) - x
+        d -= box * np.round(d / box)
+        if not len(pts) or (d ** 2).sum(1).min() > apart ** 2:
+            pts.append(x)
+            n -= 1
+    return pts
+
+
+def blob():
+    """About 120 neighbours everywhere, 250 more around the middle of the box; 136 by the mean, a buffer of 320."""
+    def ball(rng):
+        while True:
+            x = rng.uniform(-6.0, 6.0, 3)
+            if x @ x < 36.0:
+                return x + 16.0
+    rng = np.random.default_rng(4)
+    pts = _scatter(rng, 32.0, 250, ball, [], 1.0)
+    pts = _scatter(rng, 32.0, 1835, lambda g: g.uniform(0.0, 32.0, 3), pts, 1.0)
+    return I.Frame(np.array(pts), np.zeros(len(pts), dtype=np.int32), np.eye(3) * 32.0)
+
+
+def rod():
+    """320 atoms in the corner column of a 15.2 A box's three half-width cells a side, four of them next to it."""
+    rng = np.random.default_rng(4)
+    pts = _scatter(rng, 15.2, 316, lambda g: g.uniform((10.2, 10.2, 0.0), (15.1, 15.1, 15.2)), [], 0.8)
+    pts = _scatter(rng, 15.2, 4, lambda g: g.uniform((6.0, 6.0, 0.0), (9.5, 9.5, 15.2)), pts, 0.8)
+    return I.Frame(np.array(pts), np.zeros(320, dtype=np.int32), np.eye(3) * 15.2)
+
+
+def _searches(call):
+    """Names of the neighbour-search kernels that a call launches."""
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(3):  # a process's first trace can come back empty
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            call()
+            torch.cuda.synchronize()
+        names = [e.name for e in prof.events() if "k_nlist" in e.name]
+        if names:
+            break
+    return names
+
+
+@pytest.mark.parametrize("make", [blob, rod])
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+def test_uneven_density(make, precision):
+    from paper_2304_09409_gb300 import dpgb
+    fr = make()
+    m = dpgb.Model(CFG, I.make_params(CFG, 0), precision=precision, compressed=True)
+    c, t = torch.tensor(fr.coord, device="cuda"), torch.tensor(fr.atype, device="cuda")
+    ref = oracle.nlist(CFG, fr.coord, fr.atype, fr.box)
+    for _ in range(2):
+        nl = m.build_nlist(c, t, fr.box)
+        j, s = nl.export()
+        assert np.array_equal(j, ref[0].reshape(j.shape))
+        assert np.array_equal(s, ref[1].reshape(s.shape))
+        nl.free()
+    names = _searches(lambda: m.build_nlist(c, t, fr.box).free())
+    # the blob on the cell-centred search; the rod's whole-cell stream (27 times the frame) is too long for it, and
+    # takes the per-atom one with the buffer of its density, not the largest
+    assert names and all("k_nlist_cell" in n if make is blob else "k_nlist<512>" in n for n in names), names
+    if precision == "fp32":  # a call with its own list is retried the same way (1e-12: the order of FP64 additions)
+        nl = m.build_nlist(c, t, fr.box)
+        e0, f0, _, _ = m.compute(c, t, fr.box, nlist=nl)
+        other = dpgb.Model(CFG, I.make_params(CFG, 0), precision=precision, compressed=True)
+        for _ in range(4):
+            e1, f1, _, _ = other.compute(c, t, fr.box)
+            assert abs(float(e0 - e1)) <= 1e-12 * abs(float(e0))
+            assert float((f0 - f1).abs().max()) <= 1e-12 * max(float(f0.abs().max()), 1e-3)
+        nl.free()
+        other.free()
+    m.free()
