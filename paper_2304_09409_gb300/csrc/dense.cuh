@@ -27,8 +27,7 @@ struct DenseRows {
 
 // Row lists of a descriptor part: the slot rows with s != 0 (the others are padding) of every
 // (centre type, neighbour type) pair, compacted so that no layer works on padding.  Entries of pair
-// (ti, tj) start at base[ti * ntypes + tj], and there is room for cap[ti * ntypes + tj] of them; their
-// order within a pair is arbitrary.
+// (ti, tj) start at base[ti * ntypes + tj], and there is room for cap[ti * ntypes + tj] of them.
 // The room follows the per-type counts the call was set up with.  A device type array may have been rewritten
 // since those were read: that is found on the device and the call is done again, but its kernels run to the
 // end first, so entries beyond a pair's room are dropped.
@@ -40,7 +39,8 @@ struct RowLists {
 };
 
 // Append every calling thread's row (grp in [0, ngroups)) to its group's list; the whole block calls.  One
-// global atomic per block and group.
+// global atomic per block and group, so the order of a list differs from run to run: for layers whose rows
+// do not meet in a sum.
 __device__ __forceinline__ void append_row(const RowLists& rl, int ngroups, int grp, long row) {
   __shared__ int s_cnt[kMaxDenseGroups], s_base[kMaxDenseGroups];
   for (int e = threadIdx.x; e < ngroups; e += blockDim.x) s_cnt[e] = 0;
