@@ -1434,9 +1434,6 @@ int launch_mom(const DeviceModel& m, const MomArgs& g, int tiles, int which, boo
       if (bwd_smem(g, NPASS, 4) <= 226 * 1024) {
         S = 4;
         kernel = k_mom_bwd<NPASS, NPAD, 4>;
-      } else if (bwd_smem(g, NPASS, 3) > 226 * 1024) {  // lists of more than 1,000 slots
-        S = 2;
-        kernel = k_mom_bwd<NPASS, NPAD, 2>;
       }
     }
     const size_t sm = bwd_smem(g, NPASS, S);
@@ -1472,7 +1469,8 @@ int mom_npad_of(int M) {
 bool mom_supported(const DeviceModel& m) {
   int nc = 0;
   for (int t = 0; t < m.cfg.ntypes; ++t) nc += m.cfg.sel[t];
-  // the run lists of a tile's 32 atoms stay in shared memory beside the operand rings
+  // the run lists of a tile's 32 atoms stay in shared memory beside the operand rings: 512 slots (32 KB) leave
+  // the three-pass backward three stages
   return m.compressed && (m.precision == DP_PREC_FP32 || m.precision == DP_PREC_BF16) && mom_npad_of(m.M) > 0 &&
          m.A <= 16 && (m.M * m.A) % 4 == 0 && nc <= 512;
 }
@@ -1528,8 +1526,7 @@ int run_mom(const DeviceModel& m, const PathConst& pc, const PathIO& io, Arena& 
   float4* slot = ar.get<float4>(slots);
   const int ncl = (pc.nc + 7) & ~7;
   short* run_l = ar.get<short>(N * ncl);
-  // (lists of more slots than the search keeps per type leave no room for the schedule's entries)
-  uint2* run_mask = m.mom_lcp <= 256 && pc.nc <= 1024 ? ar.get<uint2>(N * pc.ntypes) : nullptr;
+  uint2* run_mask = m.mom_lcp <= 256 ? ar.get<uint2>(N * pc.ntypes) : nullptr;  // 64 bits of four intervals
   // run moments (forward) and run P (backward) share one buffer: the moments are dead by then
   void* runs = ar.get<float4>(slots * 8 > slots * 4 * parts ? slots * 8 : slots * 4 * parts);
   const long max_tiles = (N + kAtoms - 1) / kAtoms + pc.ntypes;  // every type's last tile may be short
