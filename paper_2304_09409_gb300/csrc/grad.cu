@@ -494,7 +494,7 @@ void launch_wgrad(const DenseRows& rows, const DenseShape& sh, const R* X, const
   for (int k = 0; k < rows.ngroups; ++k) {
     int n = rows.list ? listed : 4096;
     if (!rows.list)
-      while (n > 512 && tiles * nb(rows.g[k].nrows, n) < 2L * 152) n /= 2;
+      while (n > 512 && tiles * nb(rows.g[k].nrows, n) < 2L * sm_count()) n /= 2;
     g.slab_rows[k] = n;
     g.slab0[k] = at;
     at += (rows.g[k].nrows + n - 1) / n;
