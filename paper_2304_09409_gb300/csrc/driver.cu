@@ -5,7 +5,7 @@
 // Frames are concatenated; every per-atom kernel is frame-agnostic except for the frame's
 // cell (neighbour search, image shifts), which it reads from small per-frame tables uploaded
 // once per call from pinned host memory.  Per-frame energy and virial are FP64 sums of the
-// per-atom values over fixed 512-atom chunks (deterministic order), then over each frame's
+// per-atom values over fixed 128-atom chunks (deterministic order), then over each frame's
 // chunks.
 #include <algorithm>
 #include <cstring>

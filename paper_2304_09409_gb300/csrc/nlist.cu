@@ -884,8 +884,9 @@ __global__ void __launch_bounds__(kCellWarps * 32, CAP <= 256 ? 4 : 3)
       __syncwarp();
       // ---- bucket order of the surviving FP32 keys ----
       // Counting sort into NB buckets of the keys' range, in place: counts, exclusive scan, scatter of keys
-      // and stream positions through registers; afterwards bucket b ends at end_of(b).  The counting pass first settles the entries within the FP32 error of r_c by the
-      // exact FP64 test (dropped entries get the key +inf and no bucket).
+      // and stream positions through registers; afterwards bucket b ends at end_of(b).  The counting pass
+      // first settles the entries within the FP32 error of r_c by the exact FP64 test (dropped entries get
+      // the key +inf and no bucket).
       for (int b = lane; b < NB / 2; b += 32) hist[b] = 0;
       __syncwarp();
       int removed = 0;
