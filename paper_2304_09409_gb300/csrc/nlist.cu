@@ -1281,14 +1281,14 @@ int host_geometry(const dp_model_config& cfg, int natoms, const double* box, con
       // Half-width cells where whole ones fit the box badly: a box of 1.9 r_c has one cell a side and its
       // atoms test 27 boxes full of candidates, 5.8 times as many as with r_c / 2 cells.  Where the grids fit
       // more alike the wider cells serve more centre atoms per staged stream.  Steps with whole and with half cells:
-      // metal (r_c 8, 5.3 atoms a half cell) at a ratio of 5.8 356 and 267 us, 2.43 341 and 324, 2.30 562 and 541,
-      // 2.13 880 and 886, 1.73 303 and 316; water (r_c 6, 3.0 atoms) at 5.8 263 and 256, 2.73 250 and 246, 2.57 313 and
-      // 318, 2.20 444 and 467, 2.07 574 and 617: cells of few atoms, of which a block's warps have nothing to
-      // share, pay at a higher ratio.
+      // metal (r_c 8, 5.3 atoms a half cell) at a ratio of 5.8 356 and 267 us, 2.43 341 and 324, 2.14 507 and 484,
+      // 1.90 568 and 548, 1.84 974 and 1,002, 1.73 303 and 316; water (r_c 6, 3.0 atoms) at 5.8 263 and 256, 2.73 250
+      // and 246, 2.57 313 and 318, 2.20 444 and 467, 2.07 574 and 617: cells of few atoms, of which a block's
+      // warps have nothing to share, pay at a higher ratio.
       int n2[3], K2[3];
       const double span2 = grid(2, n2, K2);
       const long noff2 = (2L * K2[0] + 1) * (2 * K2[1] + 1) * (2 * K2[2] + 1);
-      const double line = natoms >= 4.0 * n2[0] * n2[1] * n2[2] ? 2.2 : 2.6;
+      const double line = natoms >= 4.0 * n2[0] * n2[1] * n2[2] ? 1.8 : 2.6;
       if (span >= line * span2 && noff2 * cfg.ntypes <= kMaxRanges)
         for (int d = 0; d < 3; ++d) {
           g.ncell[d] = n2[d];

@@ -20,7 +20,7 @@ def _water(n):
 
 
 # model, sides, cells along x * y * z: metal boxes of 1.8, 2.3, 5.0 and 7.7 cutoffs, water boxes of 1.5 to 6.7
-CASES = [("metal", 4, 3 ** 3), ("metal", 5, 2 ** 3), ("metal", 11, 9 ** 3), ("metal", 17, 7 ** 3),
+CASES = [("metal", 4, 3 ** 3), ("metal", 5, 2 ** 3), ("metal", 11, 9 ** 3), ("metal", 17, 15 ** 3),
          ("water", 3, 3 ** 3), ("water", 4, 2 ** 3), ("water", 5, 5 ** 3), ("water", 9, 4 ** 3), ("water", 13, 6 ** 3)]
 
 
