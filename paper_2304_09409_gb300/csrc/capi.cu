@@ -243,8 +243,7 @@ int read_status(dp_model* md, cudaStream_t st, int* n_overflow) {
 }
 
 // Host-side per-type atom counts when types are on the host; else read back.
-int type_starts(const int* type_host, const int* dtype_start, const DevStatus* status, int N, int ntypes, cudaStream_t st,
-                int* out) {
+int type_starts(const int* type_host, const int* dtype_start, int N, int ntypes, cudaStream_t st, int* out) {
   if (type_host) {
     std::vector<int> cnt(ntypes, 0);
     for (int i = 0; i < N; ++i) {
@@ -258,11 +257,9 @@ int type_starts(const int* type_host, const int* dtype_start, const DevStatus* s
     for (int t = 0; t < ntypes; ++t) out[t + 1] = out[t] + cnt[t];
     return DP_OK;
   }
-  int bad = 0;
   DP_CUDA_TRY(cudaMemcpyAsync(out, dtype_start, sizeof(int) * (ntypes + 1), cudaMemcpyDeviceToHost, st));
-  DP_CUDA_TRY(cudaMemcpyAsync(&bad, &status->bad_type, sizeof(int), cudaMemcpyDeviceToHost, st));
   DP_CUDA_TRY(cudaStreamSynchronize(st));
-  if (bad || out[ntypes] != N) {
+  if (out[ntypes] != N) {  // -1: a type was out of range
     set_error("atom type outside [0, ntypes)");
     return DP_E_ARG;
   }

@@ -55,7 +55,6 @@ int read_status(dp_model* md, cudaStream_t st, int* n_overflow);
 void drop_graph(dp_model* md);
 // read_status result: the per-type atom counts differ from the ones the call was set up with
 constexpr int kStatusTypeChange = -1000;
-int type_starts(const int* type_host, const int* dtype_start, const DevStatus* status, int N, int ntypes, cudaStream_t st,
-                int* out);
+int type_starts(const int* type_host, const int* dtype_start, int N, int ntypes, cudaStream_t st, int* out);
 
 }  // namespace dpgb

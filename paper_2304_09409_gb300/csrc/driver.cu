@@ -406,7 +406,7 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
   std::memset(&chk, 0, sizeof(chk));
   bool ts_known = false;
   if (copy_type) {
-    rc = type_starts(type, nullptr, nullptr, N, m.cfg.ntypes, st, io.type_start);
+    rc = type_starts(type, nullptr, N, m.cfg.ntypes, st, io.type_start);
     if (rc != DP_OK) return rc;
     ts_known = true;
   } else if (md->ts_ptr == type && md->ts_n == N) {
@@ -484,7 +484,7 @@ int run_frames(dp_model* md, dp_nlist* nlist, int F, const int* natoms, const do
       DP_CUDA_TRY(launch_type_perm(dtype, N, m.cfg.ntypes, b.perm, b.type_start, md->status, chk, s));
     }
     if (!ts_known) {  // first call on this device type array: read the counts back (synchronises)
-      int r = type_starts(nullptr, b.type_start, md->status, N, m.cfg.ntypes, s, io.type_start);
+      int r = type_starts(nullptr, b.type_start, N, m.cfg.ntypes, s, io.type_start);
       if (r != DP_OK) return r;
       md->ts_ptr = type;
       md->ts_n = N;

@@ -229,7 +229,8 @@ __device__ __forceinline__ void block_scan_counts(const int* __restrict__ in, in
 }
 
 // Sorted entries as below, with the key starts formed in shared memory by every block (block 0
-// also writes them out for the search).
+// also writes them out for the search).  type_start ends with -1 where a type was out of range: the host reads it
+// in one copy.
 __global__ void k_fill_scan(int natoms, const int* __restrict__ cell_count, int nkeys, int* __restrict__ cell_start,
                             const int2* __restrict__ atom_key, const float4* __restrict__ atom_l,
                             const int4* __restrict__ atom_m, float4* __restrict__ sorted_l, int4* __restrict__ sorted_m,
@@ -244,7 +245,7 @@ __global__ void k_fill_scan(int natoms, const int* __restrict__ cell_count, int 
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (perm && i <= ntypes) {
     const int v = s_start[i * ncells_total];
-    type_start[i] = v;
+    type_start[i] = i == ntypes && st->bad_type ? -1 : v;
     if (chk.on && v != chk.v[i]) atomicExch(&st->type_change, 1);
   }
   if (i >= natoms) return;
@@ -266,7 +267,7 @@ __global__ void k_fill(int natoms, const int2* __restrict__ atom_key, const floa
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (perm && i <= ntypes) {
     const int v = cell_start[i * ncells_total];
-    type_start[i] = v;
+    type_start[i] = i == ntypes && st->bad_type ? -1 : v;
     if (chk.on && v != chk.v[i]) atomicExch(&st->type_change, 1);
   }
   if (i >= natoms) return;
@@ -1142,9 +1143,10 @@ __global__ void __launch_bounds__(1024)
     for (int q = 0; q < DP_MAX_TYPES; ++q)
       if (t == q && q < ntypes) perm[off[q]++] = i;
   }
-  if (bad) atomicExch(&status->bad_type, 1);
+  bad = __syncthreads_or(bad);
+  if (bad && tid == 0) atomicExch(&status->bad_type, 1);
   if (chk.on && tid <= ntypes && tstart[tid] != chk.v[tid]) atomicExch(&status->type_change, 1);
-  if (tid <= ntypes) type_start[tid] = tstart[tid];
+  if (tid <= ntypes) type_start[tid] = tid == ntypes && bad ? -1 : tstart[tid];
 }
 
 }  // namespace
