@@ -1286,11 +1286,14 @@ int host_geometry(const dp_model_config& cfg, int natoms, const double* box, con
       // metal (r_c 8, 5.3 atoms a half cell) at a ratio of 5.8 356 and 267 us, 2.43 341 and 324, 2.14 507 and 484,
       // 1.90 568 and 548, 1.84 974 and 1,002, 1.73 303 and 316; water (r_c 6, 3.0 atoms) at 5.8 263 and 256, 2.73 250
       // and 246, 2.57 313 and 318, 2.20 444 and 467, 2.07 574 and 617: cells of few atoms, of which a block's
-      // warps have nothing to share, pay at a higher ratio.
+      // warps have nothing to share, pay at a higher ratio once they are more than the chip takes at a time
+      // (four blocks an SM); fewer of them do from the lower one on, by the shorter stream (a batch with water frames
+      // of 120 and 144 atoms at 2.16 and 2.59: 1,450 and 1,429).
       int n2[3], K2[3];
       const double span2 = grid(2, n2, K2);
       const long noff2 = (2L * K2[0] + 1) * (2 * K2[1] + 1) * (2 * K2[2] + 1);
-      const double line = natoms >= 4.0 * n2[0] * n2[1] * n2[2] ? 1.8 : 2.6;
+      const long cells2 = (long)n2[0] * n2[1] * n2[2];
+      const double line = natoms < 4.0 * cells2 && cells2 > 4L * sm_count() ? 2.6 : 1.8;
       if (span >= line * span2 && noff2 * cfg.ntypes <= kMaxRanges)
         for (int d = 0; d < 3; ++d) {
           g.ncell[d] = n2[d];

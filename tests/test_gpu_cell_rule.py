@@ -1,6 +1,7 @@
 """Which cell grid the neighbour search of a frame takes: half-width cells where whole ones fit the box badly, by a line that
-is higher where a half-width cell holds fewer than four atoms (csrc/nlist.cu, host_geometry).  The grid is read from the
-launch of the cell-centred search, which has a block column per cell; the lists themselves are checked elsewhere.
+is higher where half-width cells hold fewer than four atoms and are more than four an SM (csrc/nlist.cu, host_geometry).
+The grid is read from the launch of the cell-centred search, which has a block column per cell; the lists themselves are
+checked elsewhere.
 """
 import json
 import os
@@ -21,7 +22,7 @@ def _water(n):
 
 # model, sides, cells along x * y * z: metal boxes of 1.8, 2.3, 5.0 and 7.7 cutoffs, water boxes of 1.5 to 6.7
 CASES = [("metal", 4, 3 ** 3), ("metal", 5, 2 ** 3), ("metal", 11, 9 ** 3), ("metal", 17, 15 ** 3),
-         ("water", 3, 3 ** 3), ("water", 4, 2 ** 3), ("water", 5, 5 ** 3), ("water", 9, 4 ** 3), ("water", 13, 6 ** 3)]
+         ("water", 3, 3 ** 3), ("water", 4, 2 ** 3), ("water", 5, 5 ** 3), ("water", 7, 7 ** 3), ("water", 9, 4 ** 3), ("water", 13, 6 ** 3)]
 
 
 @pytest.mark.parametrize("name,n,cells", CASES)
