@@ -141,13 +141,12 @@ __device__ __forceinline__ int mom_interval(const MomArgs& g, float s, int lcap,
 // lower and the upper four intervals of a group as blocks of their own.  With run masks only the blocks
 // that some atom of the tile has a neighbour in are scheduled (the others would add exact zeros): in
 // water the intervals between the O-H bond and everything else are empty.
-constexpr int kSchedMax = DP_MAX_TYPES * 64;
 struct Sched {
   int n;                            // blocks
   int ghi[DP_MAX_TYPES];            // no masks: largest group of each type
 };
-// entries (masks only, kSchedMax of them after the kernel's other shared memory): type << 8 | block, a
-// block being a group or 2 * group + half
+// entries (masks only, after the kernel's other shared memory, room for every block of the tables): type << 8 |
+// block, a block being a group or 2 * group + half
 template <bool HALVES>
 __device__ __forceinline__ void block_of(const Sched& sc, const unsigned short* entries, int kb, int ntypes, int& t,
                                          int& grp, int& h) {
@@ -1393,15 +1392,20 @@ __global__ void k_mom_tables(const double* __restrict__ tab, int ntypes, int one
   }
 }
 
-size_t sched_smem(const MomArgs& g) { return g.run_mask ? kSchedMax * sizeof(unsigned short) : 0; }
+// The schedule's entries.  No more than the tables have blocks: with 1 KB for any eight types the one-pass
+// backward on lists of 138 slots ran two CTAs an SM instead of three (12,288 water atoms, 30 us -> 35).
+size_t sched_smem(const MomArgs& g, bool halves) {
+  return g.run_mask ? (size_t)g.ntypes * (g.lcp / 8) * (halves ? 2 : 1) * sizeof(unsigned short) : 0;
+}
 size_t fwd_smem(const MomArgs& g, int npass, int npad, int S) {
-  return fwd_region(npass, npad, g.ncl, S) + (2 * S + 1) * 8 + 16 + 1024 + sched_smem(g);
+  return fwd_region(npass, npad, g.ncl, S) + (2 * S + 1) * 8 + 16 + 1024 +
+         sched_smem(g, npass == 1 ? MomFwd<1>::halves : MomFwd<3>::halves);
 }
 size_t bwd_smem(const MomArgs& g, int npass, int S) {
   const int parts = npass == 1 ? 1 : 2;
   const int nacc = npass == 1 ? BwdDepth<1>::acc : BwdDepth<3>::acc;
   return (size_t)parts * 2 * kABlock + S * (size_t)parts * 2 * 64 * 128 + (size_t)kAtoms * g.ncl * 2 +
-         kRows * 4 + (2 * S + 1 + 2 * nacc) * 8 + 16 + 1024 + sched_smem(g);
+         kRows * 4 + (2 * S + 1 + 2 * nacc) * 8 + 16 + 1024 + sched_smem(g, false);
 }
 
 template <int NPASS, int NPAD>

@@ -59,3 +59,32 @@ def test_one_slot_more():
     _, _, prof = _run(m, I.water_frame(0), 1)
     m.free()
     assert "mom_fwd" not in prof
+
+
+def test_one_pass_kernels_keep_three_blocks_an_sm(tmp_path):
+    """The mixed mode's moment kernels on the water lists (138 slots) leave shared memory for three blocks an SM (228 KB,
+    1 KB of them per block taken by the system)."""
+    import json
+    import os
+
+    from torch.profiler import ProfilerActivity, profile
+
+    from paper_2304_09409_gb300 import dpgb
+    cfg, fr = I.water_model(), I.water_frame(0)
+    m = dpgb.Model(cfg, I.make_params(cfg, 0), precision="bf16", compressed=True)
+    c, t = torch.tensor(fr.coord, device="cuda"), torch.tensor(fr.atype, device="cuda")
+    path, used = os.path.join(str(tmp_path), "trace.json"), {}
+    for _ in range(3):  # a process's first trace can come back empty
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            m.compute(c, t, fr.box)
+            torch.cuda.synchronize()
+        prof.export_chrome_trace(path)
+        with open(path) as f:
+            for e in json.load(f)["traceEvents"]:
+                if "k_mom_fwd" in e.get("name", "") or "k_mom_bwd" in e.get("name", ""):
+                    used[e["name"].split("<")[0].split("::")[-1]] = e["args"]["shared memory"]
+        if used:
+            break
+    m.free()
+    assert set(used) == {"k_mom_fwd", "k_mom_bwd"}
+    assert all(3 * (b + 1024) <= 228 * 1024 for b in used.values()), used
