@@ -1416,7 +1416,7 @@ int launch_mom(const DeviceModel& m, const MomArgs& g, int tiles, int which, boo
   } else if (which == 0) {
     // Three passes: with more tiles than SMs three stages where two such CTAs share an SM, else two; with
     // fewer there is nobody to share with, and six keep twice the copies in flight.
-    constexpr size_t kHalfSm = 113 * 1024, kWholeSm = 226 * 1024;
+    constexpr size_t kHalfSm = 112 * 1024, kWholeSm = 225 * 1024;
     auto kernel = k_mom_fwd<NPASS, NPAD, 2>;
     int S = 2;
     if constexpr (NPASS == 3) {
@@ -1435,7 +1435,8 @@ int launch_mom(const DeviceModel& m, const MomArgs& g, int tiles, int which, boo
     auto kernel = k_mom_bwd<NPASS, NPAD, NPASS == 3 ? 3 : 2>;
     int S = NPASS == 3 ? 3 : 2;
     if constexpr (NPASS == 3) {
-      if (bwd_smem(g, NPASS, 4) <= 226 * 1024) {
+      // (lists of 512 slots would just fit four, and take 226 KB: 32,000 copper atoms 1,169 us a step against 1,150)
+      if (bwd_smem(g, NPASS, 4) <= 225 * 1024) {
         S = 4;
         kernel = k_mom_bwd<NPASS, NPAD, 4>;
       }
